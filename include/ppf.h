@@ -210,8 +210,8 @@ ppf_status ppf_update_taps(ppf_plan_t plan, const float* taps_dev, ppf_stream_t 
  *   all its threads, then splits into two groups of 256 threads that pull
  *   narrow tiles (C <= 512) independently.  A tile runs the FIR + DFT body of
  *   a single-stream kernel: the carry kernel's at C = 1024 (FIR halo carried
- *   in registers), the generic kernel's otherwise (raw rows staged through a
- *   TMA ring).  Every beam's result equals ppf_execute's up to FP32 rounding
+ *   in registers), the row kernel's at C = 2048 and 4096, the generic kernel's
+ *   otherwise (raw rows staged through a TMA ring).  Every beam's result equals ppf_execute's up to FP32 rounding
  *   (bit-identical at C = 1024 with up to 8 taps and at C = 4096, where
  *   ppf_execute runs the same body).  Asynchronous on `stream`; no allocation.
  * ppf_beams_info -- info[0]=beams, [1]=tiles, [2]=tile samples, [3]=CTAs per SM,
@@ -283,7 +283,9 @@ const char* ppf_last_error_message(void);
  *   batches; bit 4: thread-block-cluster kernel, info[2] then counts the
  *   CTAs of whole clusters; bit 5: the cluster's CTAs push their filtered
  *   channels into the transforming CTA's shared memory; bit 6: long-tap
- *   kernel, T = 17..64, raw rows and halo streamed through a TMA ring),
+ *   kernel, T = 17..64, raw rows and halo streamed through a TMA ring;
+ *   bit 7: row kernel, C >= 1024 and C = 3*2^k with T <= 16, whose short calls
+ *   run on batches of about a quarter of info[1]),
  *   info[7]=CTAs resident per SM. */
 ppf_status ppf_plan_info(ppf_plan_t plan, int info[8]);
 

@@ -229,6 +229,10 @@ extern "C" ppf_status ppf_plan(ppf_plan_t* out, int C, int T, const float* coeff
     if (ce != cudaSuccess) return cuda_fail(ce, "ppf_plan: SM count");
     ce = cudaFuncSetAttribute(e.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, e.smem);
     if (ce != cudaSuccess) return cuda_fail(ce, "ppf_plan: shared memory attribute");
+    if (e.small_batch > 0) {
+        ce = cudaFuncSetAttribute(e.small_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, e.small_smem);
+        if (ce != cudaSuccess) return cuda_fail(ce, "ppf_plan: shared memory attribute");
+    }
     int occ = 0, grid_ctas = 0;
     if (e.cluster > 0) {
         // persistent grid: as many whole clusters as can be resident at once
@@ -345,6 +349,15 @@ static ppf_status launch_fwd(ppf_plan_t p, const void* in_dev, long long in_stri
     const int unit = p->fwd.cluster > 0 ? p->fwd.cluster : 1;      // CTAs per work unit
     a.n_streams = n_streams;
     long long grid;
+    // a call that gives each SM at most one small batch runs on those
+    const long long n_small =
+        p->fwd.small_batch > 0 && n <= p->sms * (long long)p->fwd.small_batch
+            ? n_streams * ((n + p->fwd.small_batch - 1) / p->fwd.small_batch) : p->sms + 1ll;
+    if (n_small <= p->sms) {
+        cudaError_t ce = p->fwd.small_launch(a, (int)n_small, st);
+        if (ce != cudaSuccess) return cuda_fail(ce, "ppf_execute: launch");
+        return PPF_OK;
+    }
     if ((p->fwd.variant & 4) && p->fwd.cluster == 0) {
         // carry kernel: the same number of CTAs on every stream, one wave if
         // the streams allow it (at least one CTA, at most one per batch)

@@ -8,8 +8,7 @@
 // Each CTA first pulls wide tiles from a device counter and runs each with
 // the whole CTA: at C = 1024 the body of the carry kernel (one channel pair
 // per thread, the FIR halo carried in registers, warp-local DFT stages), at
-// C >= 2048 the body of the generic kernel (raw rows and their halo staged
-// through a TMA ring).  When the wide queue is empty, the CTA splits into two
+// C >= 2048 the body of the row kernel (first DFT stage on the FIR's registers).  When the wide queue is empty, the CTA splits into two
 // groups of 256 threads, each with half of the shared memory and its own
 // named barrier, and each group pulls narrow tiles from the second counter
 // and runs them independently with the generic body.
@@ -88,6 +87,11 @@ constexpr bool class_carry() {
     }
 }
 
+// C = 2048 and 4096 (the whole CTA): the row kernel's body (24 beams of 1024 to
+// 32768 spectra, 7.4 GB in and out: 5.34 -> 3.94 ms)
+template <int CI, int TI>
+constexpr bool class_row() { return kBeamC[CI] >= 2048; }
+
 template <int CI, int TI, class GRP>
 __device__ __forceinline__ bool beam_tile(const BeamsArgs& a, const BeamDesc& d, const BeamTile& t,
                                           unsigned char* smem) {
@@ -104,7 +108,9 @@ __device__ __forceinline__ bool beam_tile(const BeamsArgs& a, const BeamDesc& d,
     fa.n_spectra = d.n_spectra;
     fa.T = d.T;
     fa.flags = a.flags;
-    if constexpr (class_carry<CI, TI>())
+    if constexpr (class_row<CI, TI>())
+        return row_range<C, TM, IN_CI8, OUT_CF32>(fa, d.in, d.out, t.lo, t.hi, smem);
+    else if constexpr (class_carry<CI, TI>())
         return carry_range<C, TM, IN_CI8, OUT_CF32, false, GRP, true>(fa, d.in, d.out, t.lo, t.hi, smem);
     else
         return fwd_range<C, TM, IN_CI8, OUT_CF32, class_threads<CI>(), GRP>(fa, d.in, d.out, t.lo, t.hi, smem);
@@ -122,7 +128,8 @@ __device__ __forceinline__ bool beam_dispatch(int cls, const BeamsArgs& a, const
 
 template <int CI, int TI>
 constexpr int class_smem_of() {
-    if constexpr (class_carry<CI, TI>()) return CarryShape<kBeamC[CI], kBeamTM[TI], IN_CI8>::SMEM;
+    if constexpr (class_row<CI, TI>()) return RowShape<kBeamC[CI], kBeamTM[TI], IN_CI8>::SMEM;
+    else if constexpr (class_carry<CI, TI>()) return CarryShape<kBeamC[CI], kBeamTM[TI], IN_CI8>::SMEM;
     else return FwdShape<kBeamC[CI], kBeamTM[TI], IN_CI8, class_threads<CI>()>::SMEM;
 }
 template <int CI, int TI, int CEND>
@@ -135,7 +142,8 @@ constexpr int class_smem_max() {
 template <int CI, int TI>
 constexpr int class_batch(int cls) {
     if (cls == CI * kNumTM + TI)
-        return class_carry<CI, TI>() ? CarryShape<kBeamC[CI], kBeamTM[TI], IN_CI8>::B
+        return class_row<CI, TI>() ? RowShape<kBeamC[CI >= 5 ? CI : 5], kBeamTM[TI], IN_CI8>::B
+             : class_carry<CI, TI>() ? CarryShape<kBeamC[CI], kBeamTM[TI], IN_CI8>::B
                                      : FwdShape<kBeamC[CI], kBeamTM[TI], IN_CI8, class_threads<CI>()>::B;
     if constexpr (TI + 1 < kNumTM) return class_batch<CI, TI + 1>(cls);
     else if constexpr (CI + 1 < kNumC) return class_batch<CI + 1, 0>(cls);

@@ -366,6 +366,19 @@ __device__ __forceinline__ void cp_async(void* dst_smem, const void* src_gmem) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_addr(dst_smem)), "l"(src_gmem), "n"(BYTES)
                  : "memory");
 }
+// The same with zeros in place of the source where !ok (nothing is read then);
+// 16-byte copies bypass L1.
+template <int BYTES>
+__device__ __forceinline__ void cp_async_or_zero(void* dst_smem, const void* src_gmem, bool ok) {
+    if constexpr (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(dst_smem)), "l"(src_gmem),
+                     "r"(ok ? 16 : 0)
+                     : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(smem_addr(dst_smem)), "l"(src_gmem),
+                     "n"(BYTES), "r"(ok ? BYTES : 0)
+                     : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }

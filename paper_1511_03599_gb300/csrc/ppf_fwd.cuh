@@ -26,6 +26,8 @@
 //   and finally A_P(q) = Y[q] (q = k_0 + R_0 k_1 + ...).
 #pragma once
 
+#include <vector>
+
 #include "ppf_device.cuh"
 
 namespace ppf {
@@ -58,6 +60,14 @@ constexpr int fft_n(int C, int p) {
     for (int q = p; q < fft_stages(C); ++q) n *= fft_radix(C, q);
     return n;
 }
+// Channel counts of the row kernel (ppf_fwd_row.cuh): C = R0 * M, an R0-point
+// DFT over columns M apart, then the M-point DFT of each row in two stages of
+// row_radix; R0 = 0 elsewhere.  For C = 1024 and 3 * 2^k these are the stages
+// of the plan's own tables.
+constexpr int row_r0(int C) {
+    return C == 1024 ? 1 : C == 2048 ? 2 : is_c3(C) ? 3 : C == 4096 ? 4 : 0;
+}
+constexpr int row_radix(int C, int p) { return is_c3(C) ? fft_radix(C, p + 1) : fft_radix(1024, p); }
 // Physical index inside one spectrum slot of buffer A_p.  Buffers read by
 // a non-final stage are plain; the buffer read by the last stage (rows of
 // R = R_last elements, read column-wise by lanes walking consecutive rows
@@ -120,6 +130,14 @@ constexpr int tw_offset(int C, int p) {
     return off;
 }
 constexpr int tw_size(int C) { return tw_offset(C, fft_stages(C) - 1); }
+// The row kernel's tables: W_C^{b k0} at [(k0-1)*M + b], k0 = 1 .. R0-1, then
+// W_M^{b k} of the row's first stage (RA x RB) at [(k-1)*RB + b].  At C = 2048
+// and 4096 they follow the stage tables; elsewhere they are the stage tables.
+constexpr bool row_tw_own(int C) { return C == 2048 || C == 4096; }
+constexpr int row_tw_offset(int C) { return row_tw_own(C) ? tw_size(C) : 0; }
+constexpr int row_tw_size(int C) {
+    return row_tw_own(C) ? (row_r0(C) - 1) * (C / row_r0(C)) + (row_radix(C, 0) - 1) * row_radix(C, 1) : 0;
+}
 
 // v[k] *= W_{N_p}^{b k} for k = 1 .. R-1; tw_stage is stage p's table (NN = N_{p+1} columns)
 template <int R, int NN, bool TW_SMEM>
@@ -835,6 +853,7 @@ struct FwdInfo {
 }  // namespace ppf
 
 #include "ppf_fwd_carry.cuh"
+#include "ppf_fwd_row.cuh"
 #include "ppf_fwd_cluster.cuh"
 #include "ppf_fwd_push.cuh"
 #include "ppf_fwd_longtap.cuh"
@@ -863,12 +882,22 @@ constexpr bool carry_preferred() {
     return CarryShape<C, TM, IN>::OK && !(C == 1024 && TM > 8);
 }
 
+template <int C, int TM, int IN>
+constexpr bool row_preferred() {
+    if constexpr (row_r0(C) > 0) return RowShape<C, TM, IN>::OK && !(C == 2048 && IN == IN_CF32 && TM == 8);
+    else return false;
+}
+
 template <int C, int TM, int IN, int OUT>
 inline FwdInfo fwd_info() {
     if constexpr (carry_preferred<C, TM, IN>()) {
         using S = CarryShape<C, TM, IN>;
         return FwdInfo{S::NT, S::B, S::SMEM, fft_stages(C), TM, 1 | (S::TW_SMEM ? 2 : 0) | 4,
                        reinterpret_cast<const void*>(&pfb_fwd_carry_kernel<C, TM, IN, OUT>), 0};
+    } else if constexpr (row_preferred<C, TM, IN>()) {
+        using S = RowShape<C, TM, IN>;
+        return FwdInfo{S::NT, S::B, S::SMEM, 2 + (S::R0 > 1), TM, 128 | (S::RING ? 1 : 0) | (S::TW_SMEM ? 2 : 0),
+                       reinterpret_cast<const void*>(&pfb_fwd_row_kernel<C, TM, IN, OUT>), 0};
     } else if constexpr (PushShape<C, TM, IN>::OK && !PPF_NO_PUSH) {
         using S = PushShape<C, TM, IN>;
         return FwdInfo{S::NT, S::B, S::SMEM, fft_stages(C), TM, 1 | 2 | 4 | 16 | 32,
@@ -894,6 +923,9 @@ inline cudaError_t fwd_launch(const FwdArgs& a, int grid, cudaStream_t st) {
     if constexpr (carry_preferred<C, TM, IN>()) {
         using S = CarryShape<C, TM, IN>;
         pfb_fwd_carry_kernel<C, TM, IN, OUT><<<grid, S::NT, S::SMEM, st>>>(a);
+    } else if constexpr (row_preferred<C, TM, IN>()) {
+        using S = RowShape<C, TM, IN>;
+        pfb_fwd_row_kernel<C, TM, IN, OUT><<<grid, S::NT, S::SMEM, st>>>(a);
     } else if constexpr (PushShape<C, TM, IN>::OK && !PPF_NO_PUSH) {
         using S = PushShape<C, TM, IN>;
         pfb_fwd_push_kernel<C, TM, IN, OUT><<<grid, S::NT, S::SMEM, st>>>(a);
@@ -907,6 +939,14 @@ inline cudaError_t fwd_launch(const FwdArgs& a, int grid, cudaStream_t st) {
         using S = FwdShape<C, TM, IN>;
         pfb_fwd_kernel<C, TM, IN, OUT><<<grid, S::NT, S::SMEM, st>>>(a);
     }
+    return cudaPeekAtLastError();
+}
+
+// The row kernel's small batches (FwdEntry::small_*).
+template <int C, int TM, int IN, int OUT>
+inline cudaError_t row_small_launch(const FwdArgs& a, int grid, cudaStream_t st) {
+    using S = RowShape<C, TM, IN, 4>;
+    pfb_fwd_row_kernel<C, TM, IN, OUT, 4><<<grid, S::NT, S::SMEM, st>>>(a);
     return cudaPeekAtLastError();
 }
 
@@ -938,18 +978,29 @@ inline cudaError_t fir_launch(const FwdArgs& a, int grid, cudaStream_t st) {
 // W_{N_p}^{b k} = exp(-2 pi i b k / N_p), k = 1 .. R_p-1, at
 // [tw_offset(p) + (k-1)*N_{p+1} + b].
 // Entries of the plan's twiddle table for C.
-constexpr int tw_total_float2s(int C) { return tw_size(C); }
+constexpr int tw_total_float2s(int C) { return tw_size(C) + row_tw_size(C); }
 
+// All of them are powers of W_C; each of its C powers is evaluated once.
 template <int C>
 inline void fill_twiddles(float2* host) {
+    std::vector<float> c(C);
+    for (int e = 0; e < C; ++e) c[e] = (float)cos2pi(e, C);
+    auto power = [&](long e, int n) {                 // W_n^e, n a divisor of C; sin x = cos(x - pi/2)
+        const long i = e % n * (C / n);
+        return make_float2(c[i], -c[(i + C - C / 4) % C]);
+    };
     for (int p = 0; p + 1 < fft_stages(C); ++p) {
         const int NP = fft_n(C, p), R = fft_radix(C, p), NN = NP / R;
         for (int k = 1; k < R; ++k)
-            for (int b = 0; b < NN; ++b) {
-                const long e = (long)b * k % NP;
-                host[tw_offset(C, p) + (k - 1) * NN + b] =
-                    make_float2((float)cos2pi(e, NP), (float)(-sin2pi(e, NP)));
-            }
+            for (int b = 0; b < NN; ++b) host[tw_offset(C, p) + (k - 1) * NN + b] = power((long)b * k, NP);
+    }
+    if constexpr (row_tw_own(C)) {
+        constexpr int R0 = row_r0(C), M = C / R0, RA = row_radix(C, 0), RB = row_radix(C, 1);
+        float2* row = host + row_tw_offset(C);
+        for (int k = 1; k < R0; ++k)
+            for (int b = 0; b < M; ++b) *row++ = power((long)b * k, C);
+        for (int k = 1; k < RA; ++k)
+            for (int b = 0; b < RB; ++b) *row++ = power((long)b * k, M);
     }
 }
 

@@ -19,7 +19,14 @@ template <int TM, int IN, int OUT>
 static bool make_entry(FwdEntry* e) {
     FwdInfo i = fwd_info<PPF_C, TM, IN, OUT>();
     *e = FwdEntry{i.threads, i.batch, i.smem, i.stages, i.tap_bucket, i.variant, i.fn, &fwd_launch<PPF_C, TM, IN, OUT>,
-                  i.cluster};
+                  i.cluster, 0, 0, nullptr, nullptr};
+    if constexpr (row_preferred<PPF_C, TM, IN>()) {
+        using S = RowShape<PPF_C, TM, IN, 4>;
+        e->small_batch = S::B;
+        e->small_smem = S::SMEM;
+        e->small_fn = reinterpret_cast<const void*>(&pfb_fwd_row_kernel<PPF_C, TM, IN, OUT, 4>);
+        e->small_launch = &row_small_launch<PPF_C, TM, IN, OUT>;
+    }
     return true;
 }
 
@@ -58,7 +65,8 @@ template <int TM, int IN>
 static bool make_fir(FwdEntry* e) {
     FwdInfo i;
     if (!fir_info<PPF_C, TM, IN>(&i)) return false;
-    *e = FwdEntry{i.threads, i.batch, i.smem, i.stages, i.tap_bucket, i.variant, i.fn, &fir_launch<PPF_C, TM, IN>, 0};
+    *e = FwdEntry{i.threads, i.batch, i.smem, i.stages, i.tap_bucket, i.variant, i.fn, &fir_launch<PPF_C, TM, IN>, 0,
+                  0, 0, nullptr, nullptr};
     return true;
 }
 

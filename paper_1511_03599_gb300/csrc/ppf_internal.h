@@ -25,10 +25,15 @@ struct FwdEntry {
     int smem;        // dynamic shared memory bytes
     int stages;      // FFT stages
     int tap_bucket;  // taps rounded up to the compiled bucket
-    int variant;     // bit 0: TMA ring; bit 1: twiddles in smem; bit 2: halo carried; bit 4: cluster
+    int variant;     // bit 0: TMA ring; bit 1: twiddles in smem; bit 2: halo carried; bit 4: cluster; bit 7: row kernel
     const void* fn;  // kernel function (for occupancy queries and attributes)
     cudaError_t (*launch)(const FwdArgs&, int grid, cudaStream_t);
     int cluster;     // CTAs per thread-block cluster (0: none); grid counts CTAs
+    // the same arithmetic in smaller batches, for calls too short to give every
+    // SM one of the batches above (batch 0: none); same threads per CTA
+    int small_batch, small_smem;
+    const void* small_fn;
+    cudaError_t (*small_launch)(const FwdArgs&, int grid, cudaStream_t);
 };
 
 // Resident clusters of a cluster kernel entry (persistent grid): the most
