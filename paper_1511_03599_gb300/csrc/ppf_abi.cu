@@ -233,6 +233,10 @@ extern "C" ppf_status ppf_plan(ppf_plan_t* out, int C, int T, const float* coeff
         ce = cudaFuncSetAttribute(e.small_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, e.small_smem);
         if (ce != cudaSuccess) return cuda_fail(ce, "ppf_plan: shared memory attribute");
     }
+    if (e.short_fn != nullptr) {
+        ce = cudaFuncSetAttribute(e.short_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, e.smem);
+        if (ce != cudaSuccess) return cuda_fail(ce, "ppf_plan: shared memory attribute");
+    }
     int occ = 0, grid_ctas = 0;
     if (e.cluster > 0) {
         // persistent grid: as many whole clusters as can be resident at once
@@ -364,6 +368,11 @@ static ppf_status launch_fwd(ppf_plan_t p, const void* in_dev, long long in_stri
         const long long cps = std::max<long long>(1, std::min<long long>(p->grid / n_streams, nb));
         grid = cps * n_streams;
         if (grid > 0x7fffffffll) return fail(PPF_ERR_INVALID_ARG, "ppf_execute: too many streams");
+        if (nb <= cps * ppf::kCarryShort && p->fwd.short_launch != nullptr) {
+            cudaError_t ce = p->fwd.short_launch(a, (int)grid, st);
+            if (ce != cudaSuccess) return cuda_fail(ce, "ppf_execute: launch");
+            return PPF_OK;
+        }
     } else {
         grid = work_units(p->grid / unit, n_streams, nb) * unit;
     }

@@ -62,12 +62,14 @@ constexpr int fft_n(int C, int p) {
 }
 // Channel counts of the row kernel (ppf_fwd_row.cuh): C = R0 * M, an R0-point
 // DFT over columns M apart, then the M-point DFT of each row in two stages of
-// row_radix; R0 = 0 elsewhere.  For C = 1024 and 3 * 2^k these are the stages
+// row_radix; R0 = 0 elsewhere.  Except at C = 2048 and 4096 these are the stages
 // of the plan's own tables.
 constexpr int row_r0(int C) {
-    return C == 1024 ? 1 : C == 2048 ? 2 : is_c3(C) ? 3 : C == 4096 ? 4 : 0;
+    return C == 4096 ? 4 : is_c3(C) ? 3 : C == 2048 ? 2 : C >= 64 ? 1 : 0;
 }
-constexpr int row_radix(int C, int p) { return is_c3(C) ? fft_radix(C, p + 1) : fft_radix(1024, p); }
+constexpr int row_radix(int C, int p) {
+    return is_c3(C) ? fft_radix(C, p + 1) : fft_radix(C < 1024 ? C : 1024, p);
+}
 // Physical index inside one spectrum slot of buffer A_p.  Buffers read by
 // a non-final stage are plain; the buffer read by the last stage (rows of
 // R = R_last elements, read column-wise by lanes walking consecutive rows
@@ -884,7 +886,16 @@ constexpr bool carry_preferred() {
 
 template <int C, int TM, int IN>
 constexpr bool row_preferred() {
-    if constexpr (row_r0(C) > 0) return RowShape<C, TM, IN>::OK && !(C == 2048 && IN == IN_CF32 && TM == 8);
+    if constexpr (C >= 1024 || is_c3(C)) return RowShape<C, TM, IN>::OK && !(C == 2048 && IN == IN_CF32 && TM == 8);
+    else return false;
+}
+
+// Calls that give each SM at most one small batch (FwdEntry::small_*) run the
+// row kernel's small batches wherever the stages and the FIR order are the
+// same, so the results are too: with the row and the carry kernels.
+template <int C, int TM, int IN>
+constexpr bool row_small() {
+    if constexpr (row_preferred<C, TM, IN>() || carry_preferred<C, TM, IN>()) return RowShape<C, TM, IN, 4>::OK;
     else return false;
 }
 
@@ -947,6 +958,14 @@ template <int C, int TM, int IN, int OUT>
 inline cudaError_t row_small_launch(const FwdArgs& a, int grid, cudaStream_t st) {
     using S = RowShape<C, TM, IN, 4>;
     pfb_fwd_row_kernel<C, TM, IN, OUT, 4><<<grid, S::NT, S::SMEM, st>>>(a);
+    return cudaPeekAtLastError();
+}
+
+// The carry kernel's form for short ranges (FwdEntry::short_*).
+template <int C, int TM, int IN, int OUT>
+inline cudaError_t carry_short_launch(const FwdArgs& a, int grid, cudaStream_t st) {
+    using S = CarryShape<C, TM, IN>;
+    pfb_fwd_carry_kernel<C, TM, IN, OUT, false, true><<<grid, S::NT, S::SMEM, st>>>(a);
     return cudaPeekAtLastError();
 }
 

@@ -134,7 +134,14 @@ struct CarryShape : CarryShapeSel<C, TM, IN>::type {};
 // FIRONLY: the unfused ablation -- the FIR alone, writing the filtered
 // spectra y (complex FP32, spectrum-major) to global memory instead of
 // transforming them (the paper's FIR kernel followed by a separate DFT).
-template <int C, int TM, int IN, int OUT, bool FIRONLY, class GRP, bool MULTI>
+//
+// SHORT: for ranges of few batches.  The ring's slots start T-1 rows in (the
+// rows before are carried from the start), so a range of nb batches takes nb
+// passes; otherwise its last T-1 outputs take a pass of their own.  On long
+// ranges the shifted form measured 1-3 % slower (C = 512, int8 and int16); on
+// short ones it saves up to half the time (C = 256, T = 8, FP32, 4096 spectra,
+// two batches per CTA: 8.5 -> 6.1 us).
+template <int C, int TM, int IN, int OUT, bool FIRONLY, class GRP, bool MULTI, bool SHORT = false>
 __device__ __forceinline__ bool carry_range(const FwdArgs& args, const void* in, void* out, long long lo, long long hi,
                                             unsigned char* smem) {
     using S = CarryShape<C, TM, IN>;
@@ -157,9 +164,10 @@ __device__ __forceinline__ bool carry_range(const FwdArgs& args, const void* in,
     if (nb <= 0) return true;
     if constexpr (MULTI) GRP::sync();                // the group's previous range is done with shared memory
     const long long vlo = lo * B, vhi = (hi * B < n_spectra) ? hi * B : n_spectra;
-    const long long nraw_b = (T > 1) ? nb + 1 : nb;  // raw batches this range streams
+    const long long nraw_b = (T > 1 && !SHORT) ? nb + 1 : nb;  // raw batches this range streams
+    const int sh = SHORT ? T - 1 : 0;                // rows before the first slot
     auto rows_of = [&](long long j) -> long long {
-        const long long r = n_raw - (lo + j) * B;
+        const long long r = n_raw - sh - (lo + j) * B;
         return r <= 0 ? 0 : (r < B ? r : B);
     };
     auto issue = [&](long long j) {
@@ -170,10 +178,10 @@ __device__ __forceinline__ bool carry_range(const FwdArgs& args, const void* in,
             mbar_expect_tx(bar, bytes);
             if constexpr (PPF_TMA_EVICT_FIRST)
                 tma_load_1d_once(ring + (j & 1) * S::SLOTB,
-                                 static_cast<const unsigned char*>(in) + (size_t)(lo + j) * B * C * BIN, bytes, bar);
+                                 static_cast<const unsigned char*>(in) + (size_t)((lo + j) * B + sh) * C * BIN, bytes, bar);
             else
                 tma_load_1d(ring + (j & 1) * S::SLOTB,
-                            static_cast<const unsigned char*>(in) + (size_t)(lo + j) * B * C * BIN, bytes, bar);
+                            static_cast<const unsigned char*>(in) + (size_t)((lo + j) * B + sh) * C * BIN, bytes, bar);
         }
     };
     // fp32 input: the first two raw batches are requested before the taps,
@@ -208,11 +216,11 @@ __device__ __forceinline__ bool carry_range(const FwdArgs& args, const void* in,
             h1[t] = pk2(h.y, h.y);
         }
     }
-    // carried rows x_i = raw row lo*B - (TM-1) + i, i < TM-1 (zero before the stream)
+    // carried rows x_i = raw row lo*B + sh - (TM-1) + i, i < TM-1 (zero before the stream)
     float4 carry[TM > 1 ? TM - 1 : 1];
 #pragma unroll
     for (int i = 0; i < TM - 1; ++i) {
-        const long long r = lo * B - (TM - 1) + i;
+        const long long r = lo * B + sh - (TM - 1) + i;
         carry[i] = (r >= 0 && r < n_raw) ? load_pair_global<IN>(in, r * C + 2 * cp)
                                          : make_float4(0.f, 0.f, 0.f, 0.f);
     }
@@ -268,7 +276,7 @@ __device__ __forceinline__ bool carry_range(const FwdArgs& args, const void* in,
 #pragma unroll
             for (int i = 0; i < TM - 1; ++i) carry[i] = nxt[i];
             if constexpr (FIRONLY) {
-                const long long sb = (lo + k) * B - (T - 1);
+                const long long sb = (lo + k) * B + sh - (T - 1);
 #pragma unroll
                 for (int j = 0; j < B; ++j) {
                     const long long s = sb + j;
@@ -294,7 +302,7 @@ __device__ __forceinline__ bool carry_range(const FwdArgs& args, const void* in,
         }
         // ---------------------------------------------------------- FFT
         if constexpr (!FIRONLY) {
-            const long long sb = (lo + k) * B - (T - 1);     // output spectrum of batch row 0
+            const long long sb = (lo + k) * B + sh - (T - 1);     // output spectrum of batch row 0
             static_for<NST>([&](auto p) {
                 fft_stage<C, B, NT, decltype(p)::value, OUT, S::TW_SMEM, S::SPW, false, false, S::LAYOUT, GRP>(
                     ybuf, tws, out, sb, vlo, vhi);
@@ -309,7 +317,10 @@ __device__ __forceinline__ bool carry_range(const FwdArgs& args, const void* in,
     return true;
 }
 
-template <int C, int TM, int IN, int OUT, bool FIRONLY = false>
+// Most batches per CTA for the SHORT form.
+constexpr int kCarryShort = 16;
+
+template <int C, int TM, int IN, int OUT, bool FIRONLY = false, bool SHORT = false>
 __global__ void __launch_bounds__(CarryShape<C, TM, IN>::NT, CarryShape<C, TM, IN>::MINB)
 pfb_fwd_carry_kernel(FwdArgs args) {
     using S = CarryShape<C, TM, IN>;
@@ -322,7 +333,7 @@ pfb_fwd_carry_kernel(FwdArgs args) {
     void* out = static_cast<unsigned char*>(args.out) + (size_t)strm * args.out_stride * (OUT == OUT_CF32 ? 8 : 4);
     const long long lo = (long long)bx * nbt / cps;
     const long long hi = (long long)(bx + 1) * nbt / cps;
-    carry_range<C, TM, IN, OUT, FIRONLY, CtaGroup, false>(args, in, out, lo, hi, smem);
+    carry_range<C, TM, IN, OUT, FIRONLY, CtaGroup, false, SHORT>(args, in, out, lo, hi, smem);
 }
 
 }  // namespace ppf

@@ -19,13 +19,17 @@ template <int TM, int IN, int OUT>
 static bool make_entry(FwdEntry* e) {
     FwdInfo i = fwd_info<PPF_C, TM, IN, OUT>();
     *e = FwdEntry{i.threads, i.batch, i.smem, i.stages, i.tap_bucket, i.variant, i.fn, &fwd_launch<PPF_C, TM, IN, OUT>,
-                  i.cluster, 0, 0, nullptr, nullptr};
-    if constexpr (row_preferred<PPF_C, TM, IN>()) {
+                  i.cluster, 0, 0, nullptr, nullptr, nullptr, nullptr};
+    if constexpr (row_small<PPF_C, TM, IN>()) {
         using S = RowShape<PPF_C, TM, IN, 4>;
         e->small_batch = S::B;
         e->small_smem = S::SMEM;
         e->small_fn = reinterpret_cast<const void*>(&pfb_fwd_row_kernel<PPF_C, TM, IN, OUT, 4>);
         e->small_launch = &row_small_launch<PPF_C, TM, IN, OUT>;
+    }
+    if constexpr (carry_preferred<PPF_C, TM, IN>()) {
+        e->short_fn = reinterpret_cast<const void*>(&pfb_fwd_carry_kernel<PPF_C, TM, IN, OUT, false, true>);
+        e->short_launch = &carry_short_launch<PPF_C, TM, IN, OUT>;
     }
     return true;
 }
@@ -66,7 +70,7 @@ static bool make_fir(FwdEntry* e) {
     FwdInfo i;
     if (!fir_info<PPF_C, TM, IN>(&i)) return false;
     *e = FwdEntry{i.threads, i.batch, i.smem, i.stages, i.tap_bucket, i.variant, i.fn, &fir_launch<PPF_C, TM, IN>, 0,
-                  0, 0, nullptr, nullptr};
+                  0, 0, nullptr, nullptr, nullptr, nullptr};
     return true;
 }
 

@@ -34,6 +34,9 @@ struct FwdEntry {
     int small_batch, small_smem;
     const void* small_fn;
     cudaError_t (*small_launch)(const FwdArgs&, int grid, cudaStream_t);
+    // carry kernel: the form for at most kCarryShort batches per CTA (nullptr: none)
+    const void* short_fn;
+    cudaError_t (*short_launch)(const FwdArgs&, int grid, cudaStream_t);
 };
 
 // Resident clusters of a cluster kernel entry (persistent grid): the most
