@@ -253,9 +253,8 @@ extern "C" ppf_status ppf_plan(ppf_plan_t* out, int C, int T, const float* coeff
         grid_ctas = sms * occ;
     }
 
-    // Device tables: taps padded to the bucket with zero rows (and 4 more zero
-    // rows for the largest bucket: the long-tap kernel loads taps 4 ahead), twiddles.
-    std::vector<float> taps((size_t)(tm == PPF_MAX_TAPS ? tm + 4 : tm) * C, 0.f);
+    // Device tables: taps padded to the bucket with zero rows, twiddles.
+    std::vector<float> taps((size_t)tm * C, 0.f);
     std::memcpy(taps.data(), coeffs_host, sizeof(float) * (size_t)C * T);
     std::vector<float> tw;
     twiddles(C, tw);

@@ -353,6 +353,22 @@ __device__ __forceinline__ void tma_load_1d_once(void* dst_smem, const void* src
         "l"(src_gmem), "r"(bytes), "r"(smem_addr(bar)), "l"(pol)
         : "memory");
 }
+// One box of a tensor map global -> shared (tile mode) completing on `bar`;
+// the smem address is 128-byte aligned, x * element size a multiple of 16.
+__device__ __forceinline__ void tma_load_box2(void* dst_smem, const void* map, int x, int y, uint64_t* bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
+            smem_addr(dst_smem)),
+        "l"(map), "r"(x), "r"(y), "r"(smem_addr(bar))
+        : "memory");
+}
+__device__ __forceinline__ void tma_load_box3(void* dst_smem, const void* map, int x, int y, int z, uint64_t* bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::
+            "r"(smem_addr(dst_smem)),
+        "l"(map), "r"(x), "r"(y), "r"(z), "r"(smem_addr(bar))
+        : "memory");
+}
 // Hint: bring a global range into L2 ahead of its use (bytes multiple of 16).
 __device__ __forceinline__ void tma_prefetch_l2(const void* src_gmem, uint32_t bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src_gmem), "r"(bytes) : "memory");

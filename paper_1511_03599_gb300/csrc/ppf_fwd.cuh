@@ -944,8 +944,7 @@ inline cudaError_t fwd_launch(const FwdArgs& a, int grid, cudaStream_t st) {
         using S = ClusterShape<C, TM, IN>;
         pfb_fwd_cluster_kernel<C, TM, IN, OUT><<<grid, S::NT, S::SMEM, st>>>(a);
     } else if constexpr (TM == 64 && LongShape<C, IN>::OK && !PPF_NO_LONGTAP) {
-        using S = LongShape<C, IN>;
-        pfb_fwd_longtap_kernel<C, IN, OUT><<<grid, S::NT, S::SMEM, st>>>(a);
+        return longtap_launch<C, IN, OUT, 1>(a, grid, st);
     } else {
         using S = FwdShape<C, TM, IN>;
         pfb_fwd_kernel<C, TM, IN, OUT><<<grid, S::NT, S::SMEM, st>>>(a);

@@ -27,6 +27,15 @@ static bool make_entry(FwdEntry* e) {
         e->small_fn = reinterpret_cast<const void*>(&pfb_fwd_row_kernel<PPF_C, TM, IN, OUT, 4>);
         e->small_launch = &row_small_launch<PPF_C, TM, IN, OUT>;
     }
+    if constexpr (TM == 64) {
+        if constexpr (LongShape<PPF_C, IN>::OK) {
+            using S = LongShape<PPF_C, IN, 2>;
+            e->small_batch = S::B;
+            e->small_smem = S::SMEM;
+            e->small_fn = reinterpret_cast<const void*>(&pfb_fwd_longtap_kernel<PPF_C, IN, OUT, 2>);
+            e->small_launch = &longtap_launch<PPF_C, IN, OUT, 2>;
+        }
+    }
     if constexpr (carry_preferred<PPF_C, TM, IN>()) {
         e->short_fn = reinterpret_cast<const void*>(&pfb_fwd_carry_kernel<PPF_C, TM, IN, OUT, false, true>);
         e->short_launch = &carry_short_launch<PPF_C, TM, IN, OUT>;
