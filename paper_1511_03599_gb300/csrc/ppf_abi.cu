@@ -442,28 +442,10 @@ static ppf_status backward_unfused(ppf_plan_t p, const void* grad_out_dev, const
                                            (n_spectra + p->idft.batch - 1) / p->idft.batch);
     ce = p->idft.launch(ia, (int)idft_grid, st);
     if (ce != cudaSuccess) return cuda_fail(ce, "ppf_backward: inverse DFT launch");
-    if (grad_in_dev != nullptr) {
-        ppf::AdjFirArgs fa;
-        fa.gy = p->d_gy;
-        fa.taps = p->d_taps;
-        fa.gx = static_cast<float2*>(grad_in_dev);
-        fa.n_spectra = n_spectra;
-        fa.n_streams = n_streams;
-        fa.gx_stride = n_raw * C;
-        fa.C = C;
-        fa.T = T;
-        const long long tiles = n_streams * ((n_raw + ppf::kAdjL - 1) / ppf::kAdjL);
-        const long long pair_blocks = (C / 2 + 127) / 128;
-        const long long gx_grid = std::min<long long>(tiles, std::max<long long>(1, 16LL * p->sms / pair_blocks));
-        ce = ppf::bwd_gradx(fa, (int)gx_grid, st);
-        if (ce != cudaSuccess) return cuda_fail(ce, "ppf_backward: grad_in launch");
-    }
+    // parts of the row tiles of all streams, one CTA per part and channel block;
+    // partial sums capped at 2^25 floats
+    long long parts = ppf::bwd_grad_parts((int)p->in, C, T, p->sms, n_raw, n_streams);
     if (grad_taps_dev != nullptr) {
-        // parts of the rows of all streams: about 8 CTAs per SM in all, at
-        // least 64 rows per part, partial sums capped at 2^25 floats
-        const long long blocks = ((C / 2 + 127) / 128) * (long long)ppf::bwd_gradh_tap_blocks(T);
-        long long parts = std::max<long long>(1, (8LL * p->sms + blocks - 1) / blocks);
-        parts = std::min<long long>(parts, std::max<long long>(1, n_streams * n_spectra / 64));
         parts = std::min<long long>(parts, std::max<long long>(1, (1LL << 25) / ((long long)TM * C)));
         if (parts > p->partials_ctas) {
             if (p->d_partials) cudaFree(p->d_partials);
@@ -473,19 +455,19 @@ static ppf_status backward_unfused(ppf_plan_t p, const void* grad_out_dev, const
             if (ce != cudaSuccess) return cuda_fail(ce, "ppf_backward: partial sums");
             p->partials_ctas = parts;
         }
-        ppf::AdjCorrArgs ca;
-        ca.gy = p->d_gy;
-        ca.x = in_dev;
-        ca.partials = p->d_partials;
-        ca.n_spectra = n_spectra;
-        ca.n_streams = n_streams;
-        ca.x_stride = n_raw * C;
-        ca.C = C;
-        ca.T = T;
-        ca.TM = TM;
-        ca.n_parts = (int)parts;
-        ce = ppf::bwd_gradh((int)p->in, ca, st);
-        if (ce != cudaSuccess) return cuda_fail(ce, "ppf_backward: grad_taps launch");
+    }
+    ppf::AdjArgs ga;
+    ga.gx = static_cast<float2*>(grad_in_dev);
+    ga.partials = grad_taps_dev != nullptr ? p->d_partials : nullptr;
+    ga.err = p->d_err;
+    ga.n_spectra = n_spectra;
+    ga.n_streams = n_streams;
+    ga.C = C;
+    ga.T = T;
+    ga.TM = TM;
+    ce = ppf::bwd_grad((int)p->in, ga, p->d_gy, in_dev, p->d_taps, (int)parts, st);
+    if (ce != cudaSuccess) return cuda_fail(ce, "ppf_backward: gradient launch");
+    if (grad_taps_dev != nullptr) {
         ce = ppf::bwd_reduce(p->d_partials, (int)parts, T, TM, C, p->d_err, grad_taps_dev, st);
         if (ce != cudaSuccess) return cuda_fail(ce, "ppf_backward: tap-gradient reduction");
     }

@@ -2,6 +2,8 @@
 // int16 / FP32 input, C in {64, 128, 256, 512}, tap buckets up to 16 where
 // the batch holds the halo) and the runtime-shape passes of the unfused
 // adjoint, and exports their lookups and launches.
+#include <algorithm>
+
 #include "ppf_bwd.cuh"
 #include "ppf_bwd_unfused.cuh"
 #include "ppf_internal.h"
@@ -51,28 +53,63 @@ bool bwd_lookup(int C, int tm, int in, BwdEntry* e) {
 cudaError_t bwd_reduce(const float* partials, int nparts, int T, int TM, int C, const int* err, float* grad_h,
                        cudaStream_t st) {
     const int TC = T * C;
-    pfb_bwd_reduce_kernel<<<(TC + 255) / 256, 256, 0, st>>>(partials, nparts, TC, TM * C, err, grad_h);
+    pfb_bwd_reduce_kernel<<<(TC + 31) / 32, dim3(32, kReduceLanes), 0, st>>>(partials, nparts, TC, TM * C, err, grad_h);
     return cudaPeekAtLastError();
 }
 
-cudaError_t bwd_gradx(const AdjFirArgs& a, int grid_x, cudaStream_t st) {
-    const int pairs = a.C / 2, nt = pairs < 128 ? pairs : 128;
-    pfb_bwd_gradx_kernel<<<dim3(grid_x, (pairs + nt - 1) / nt), nt, 0, st>>>(a);
+template <int IN, int NCT, bool GX, bool GH>
+static cudaError_t grad_launch(const AdjArgs& a, const AdjMaps& m, int parts, cudaStream_t st) {
+    using S = AdjShape<IN, NCT>;
+    const int smem = S::smem(GH ? a.T : 0);
+    const cudaError_t ce = cudaFuncSetAttribute(pfb_bwd_grad_kernel<IN, NCT, GX, GH>,
+                                                cudaFuncAttributeMaxDynamicSharedMemorySize, S::smem(PPF_MAX_TAPS));
+    if (ce != cudaSuccess) return ce;
+    pfb_bwd_grad_kernel<IN, NCT, GX, GH><<<dim3(parts, a.C / NCT), S::NT, smem, st>>>(a, m.g, m.x, m.taps);
     return cudaPeekAtLastError();
 }
 
-int bwd_gradh_tap_blocks(int T) { return (T + kAdjTB - 1) / kAdjTB; }
+template <int IN, int NCT>
+static cudaError_t grad_by_sums(const AdjArgs& a, const AdjMaps& m, int parts, cudaStream_t st) {
+    if (a.gx == nullptr) return grad_launch<IN, NCT, false, true>(a, m, parts, st);
+    if (a.partials == nullptr) return grad_launch<IN_CI8, NCT, true, false>(a, m, parts, st);   // x is not read
+    return grad_launch<IN, NCT, true, true>(a, m, parts, st);
+}
 
-cudaError_t bwd_gradh(int in, const AdjCorrArgs& a, cudaStream_t st) {
-    const int pairs = a.C / 2, nt = pairs < 128 ? pairs : 128;
-    const dim3 grid(a.n_parts, (pairs + nt - 1) / nt, bwd_gradh_tap_blocks(a.T));
+template <int IN>
+static cudaError_t grad_by_channels(const AdjArgs& a, const AdjMaps& m, int parts, cudaStream_t st) {
+    return a.C == 32 ? grad_by_sums<IN, 32>(a, m, parts, st)
+         : a.C == 64 ? grad_by_sums<IN, 64>(a, m, parts, st) : grad_by_sums<IN, 128>(a, m, parts, st);
+}
+
+// Channels per CTA (every planned C >= 128 is a multiple of 128).
+static int grad_channels(int C) { return C < 128 ? C : 128; }
+
+int bwd_grad_parts(int in, int C, int T, int sms, long long n_raw, long long n_streams) {
+    const int nct = grad_channels(C), blocks = C / nct;
+    // resident CTAs: bounded by registers (AdjShape::MINB) and by the grad_h table
+    const int regs = nct == 128 ? 3 : nct == 64 ? 5 : 8;
+    const int bytes = (in == IN_CF32 ? AdjShape<IN_CF32, 128>::smem(T) : AdjShape<IN_CI8, 128>::smem(T)) / 128 * nct + 1024;
+    const int fit = 228 * 1024 / bytes;
+    const long long tiles = n_streams * ((n_raw + kAdjL - 1) / kAdjL);
+    const long long parts = std::max(1ll, (long long)sms * std::max(1, std::min(regs, fit)) / blocks);
+    return (int)std::min(parts, tiles);
+}
+
+cudaError_t bwd_grad(int in, const AdjArgs& a, const float2* gy, const void* x, const float* taps, int parts,
+                     cudaStream_t st) {
+    AdjMaps m;
+    const int nct = grad_channels(a.C), bin = in == IN_CI8 ? 2 : in == IN_CI16 ? 4 : 8;
+    const unsigned long long C = a.C, S = a.n_spectra, n_raw = S + a.T - 1;
+    cudaError_t ce = make_tmap(&m.g, gy, 8, C, S, C * 8, a.n_streams, S * C * 8, nct, kAdjRC);
+    if (ce == cudaSuccess) ce = make_tmap(&m.x, x, bin, C, n_raw, C * bin, a.n_streams, n_raw * C * bin, nct, kAdjRC);
+    if (ce == cudaSuccess) ce = make_tmap(&m.taps, taps, 4, C, a.TM, C * 4, 0, 0, nct, kAdjRC);
+    if (ce != cudaSuccess) return ce;
     switch (in) {
-        case IN_CI8: pfb_bwd_gradh_kernel<IN_CI8><<<grid, nt, 0, st>>>(a); break;
-        case IN_CI16: pfb_bwd_gradh_kernel<IN_CI16><<<grid, nt, 0, st>>>(a); break;
-        case IN_CF32: pfb_bwd_gradh_kernel<IN_CF32><<<grid, nt, 0, st>>>(a); break;
+        case IN_CI8: return grad_by_channels<IN_CI8>(a, m, parts, st);
+        case IN_CI16: return grad_by_channels<IN_CI16>(a, m, parts, st);
+        case IN_CF32: return grad_by_channels<IN_CF32>(a, m, parts, st);
         default: return cudaErrorInvalidValue;
     }
-    return cudaPeekAtLastError();
 }
 
 }  // namespace ppf

@@ -295,20 +295,29 @@ __global__ void __launch_bounds__(BwdShape<C, TM, IN>::NT, 1) pfb_bwd_kernel(Bwd
     }
 }
 
-// grad_h[t*C + c] = sum over CTAs, in CTA order, of the partial sums.  When
+// grad_h[t*C + c] = sum of the partial sums over CTAs.  kReduceLanes threads per
+// element each sum every kReduceLanes-th row, in order, and the first adds their
+// sums in order (deterministic).  One thread per element read its 150 - 450
+// rows in a chain of loads on 16 CTAs: 13 us at C = 512, T = 8, now 3.  When
 // the status word is set (a bounded wait of the adjoint gave up, so some
 // partial rows were never written), every element is NaN instead.
-static __global__ void pfb_bwd_reduce_kernel(const float* __restrict__ partials, int nparts, int TC, int TMC,
-                                      const int* __restrict__ err, float* __restrict__ grad_h) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= TC) return;
-    if (*err != 0) {
-        grad_h[i] = __int_as_float(0x7fc00000);
-        return;
-    }
+constexpr int kReduceLanes = 16;
+static __global__ void __launch_bounds__(32 * kReduceLanes)
+pfb_bwd_reduce_kernel(const float* __restrict__ partials, int nparts, int TC, int TMC, const int* __restrict__ err,
+                      float* __restrict__ grad_h) {
+    __shared__ float sums[kReduceLanes][32];
+    const int i = blockIdx.x * 32 + threadIdx.x;
     float s = 0.f;
-    for (int p = 0; p < nparts; ++p) s += partials[(size_t)p * TMC + i];
-    grad_h[i] = s;
+    if (i < TC) {
+#pragma unroll 8
+        for (int p = threadIdx.y; p < nparts; p += kReduceLanes) s += partials[(size_t)p * TMC + i];
+    }
+    sums[threadIdx.y][threadIdx.x] = s;
+    __syncthreads();
+    if (threadIdx.y == 0 && i < TC) {
+        for (int q = 1; q < kReduceLanes; ++q) s += sums[q][threadIdx.x];
+        grad_h[i] = *err != 0 ? __int_as_float(0x7fc00000) : s;
+    }
 }
 
 struct BwdInfo {

@@ -12,22 +12,16 @@
 //   1. pfb_bwd_idft_kernel<C>: batches of G rows through shared memory, the
 //      forward's DFT stages in their inverse mode (conj(F conj(.))), g_y rows
 //      to the scratch;
-//   2. pfb_bwd_gradx_kernel: one thread per channel pair and tile of kAdjL
-//      raw rows, taps outermost with a window of kAdjL g_y rows in registers
-//      (one new row per tap, with its tap, staged kAdjStage taps ahead);
-//   3. pfb_bwd_gradh_kernel<IN>: one thread per channel pair, block of
-//      kAdjTB taps and part of the rows of all streams, a window of kAdjTB
-//      x rows in registers (one new x row and one g_y row per row, staged
-//      kAdjStage rows ahead); per-part partial sums reduced in a fixed order
-//      by pfb_bwd_reduce_kernel (deterministic).
-// The staging: each thread copies the rows it will need with cp.async into
-// shared-memory slots of its own and waits for the oldest group, so several
-// global loads are in flight per thread without holding registers.
-// HBM traffic per raw sample is about G 8 + g_y 8 (write) + g_y 8 + grad_x 8
-// + g_y 8 + x; the halo and tap-block re-reads come from L2.
+//   2. pfb_bwd_grad_kernel<IN>: both other sums from one pass over g_y, one
+//      thread per channel, a window of kAdjL rows of g_y in registers, rows,
+//      samples and taps through a TMA ring; per-part partial sums of grad_h
+//      reduced in a fixed order by pfb_bwd_reduce_kernel (deterministic).
+// HBM traffic per raw sample is about G 8 + g_y 8 (write) + g_y 8 + grad_x 8 + x;
+// the halo re-reads come from L2.
 #pragma once
 
 #include "ppf_fwd.cuh"
+#include "ppf_tmap.h"
 
 namespace ppf {
 
@@ -81,205 +75,233 @@ __global__ void __launch_bounds__(IdftShape<C>::NT) pfb_bwd_idft_kernel(IdftArgs
     }
 }
 
-struct AdjFirArgs {
-    const float2* gy;        // g_y, n_spectra*C per stream, streams contiguous
-    const float* taps;       // tap-major, rows >= T zero
-    float2* gx;              // grad_x, n_raw*C per stream, streams gx_stride apart
-    long long n_spectra, n_streams, gx_stride;
-    int C, T;
+// grad_x and the tap correlation in one pass over g_y.  A CTA owns NCT channels
+// (one per consumer thread) and a share of the tiles of kAdjL raw rows of all
+// streams.  For the tile at raw row r0 a window of kAdjL rows of g_y lives in
+// registers; step u (tap t = T-1-u) has rows r0 + j - t, j = 0 .. kAdjL-1, in it,
+// so both sums need no other operand:
+//   grad_x[r0+j] += h[t] g_y[r0+j-t]                  (kAdjL packed FMAs)
+//   grad_h[t]    += sum_j Re(conj(g_y[r0+j-t]) x[r0+j])  (kAdjL packed FMAs)
+// then the oldest row leaves the window and row r0 + kAdjL - t enters.  The sum
+// over j is added to the thread's column of a [T][NCT] table in shared memory,
+// written out once per CTA (partial sums, reduced in a fixed order later).
+// A producer warp keeps a ring of chunks filled with boxes of tensor maps: 8
+// rows of g_y with 8 rows of x (the window and the tile's samples), then 8
+// rows of g_y with 8 taps.  Rows outside a stream read as zeros.
+// Bound by FP32 issue (2 T packed FMAs per sample, 1.0 clock per sample and SM at
+// T = 32; it takes 2.2, 52 % of the FMA pipe) and for few taps by HBM.  The two
+// kernels it replaces read g_y once each, the halo five times from L2 (tiles
+// of 8 rows), and spent as many instructions on staging as on FMAs: C = 512,
+// T = 32, int8, 65536 spectra 457 -> 236 us; the whole adjoint (GS/s) C = 512
+// T = 64 33 -> 60, C = 1024 T = 8 FP32 98 -> 128, C = 32 T = 8 50 -> 99.
+constexpr int kAdjL = 16;    // raw rows per tile
+constexpr int kAdjRC = 8;    // rows (and taps) per chunk
+constexpr int kAdjNS = 3;    // ring slots
+
+struct AdjArgs {
+    float2* gx;              // grad_x, n_raw*C per stream, streams contiguous (GX)
+    float* partials;         // gridDim.x rows of TM*C partial sums (GH)
+    int* err;
+    long long n_spectra, n_streams;
+    int C, T, TM;
 };
 
-constexpr int kAdjL = 8;     // raw rows per grad_x tile
-constexpr int kAdjStage = 8; // rows (or taps) each thread has in flight through its staging slots
-constexpr int kAdjTB = 8;    // taps per grad_h block
+struct AdjMaps {
+    CUtensorMap g, x, taps;
+};
 
-// Complex pair (2 channels) as (re0, re1) and (im0, im1) packed registers.
-__device__ __forceinline__ void load_gpair(const float2* __restrict__ row, int p, bool ok, unsigned long long& re,
-                                           unsigned long long& im) {
-    const float4 v = ok ? __ldg(reinterpret_cast<const float4*>(row) + p) : make_float4(0.f, 0.f, 0.f, 0.f);
-    re = pk2(v.x, v.z);
-    im = pk2(v.y, v.w);
-}
+template <int IN, int NCT>
+struct AdjShape {
+    static constexpr int NT = NCT + 32;
+    static constexpr int MINB = NCT == 128 ? 3 : NCT == 64 ? 5 : 8;  // CTAs per SM: at most 16 warps of 128 registers
+    static constexpr int BIN = InTraits<IN>::bytes;
+    static constexpr int GB = kAdjRC * NCT * 8;                      // a chunk's rows of g_y
+    static constexpr int XB = kAdjRC * NCT * (BIN > 4 ? BIN : 4);    // its rows of x, or its taps
+    static constexpr int CHUNKB = GB + XB;
+    static constexpr int BAR_OFF = kAdjNS * CHUNKB;
+    static constexpr int GH_OFF = BAR_OFF + 64;
+    static constexpr int smem(int T) { return GH_OFF + T * NCT * 4; }
+};
 
-// grid.x: tiles (grid-stride over n_streams * ceil(n_raw / kAdjL)), grid.y: blocks of channel pairs.  Each thread
-// streams the g_y rows its taps bring in, and the taps, through kAdjStage
-// shared-memory staging slots of its own (cp.async), kAdjStage taps ahead.
-static __global__ void __launch_bounds__(128) pfb_bwd_gradx_kernel(AdjFirArgs a) {
-    constexpr int L = kAdjL, D = kAdjStage;
-    static_assert(L % D == 0, "staging slots repeat within a tap block");
-    __shared__ __align__(16) float4 sg[D][128];                      // g_y pair of a staged row
-    __shared__ __align__(8) float2 sh[D][128];                       // taps of the pair for a staged tap
-    const int C = a.C, T = a.T;
-    const int tl = threadIdx.x;
-    const int p = blockIdx.y * blockDim.x + tl;                      // channel pair
-    if (p >= C / 2) return;
-    const long long S = a.n_spectra, n_raw = S + T - 1;
+template <int IN, int NCT, bool GX, bool GH>
+__global__ void __launch_bounds__(AdjShape<IN, NCT>::NT, AdjShape<IN, NCT>::MINB)
+pfb_bwd_grad_kernel(AdjArgs a, const __grid_constant__ CUtensorMap g_map, const __grid_constant__ CUtensorMap x_map,
+                    const __grid_constant__ CUtensorMap tap_map) {
+    using S = AdjShape<IN, NCT>;
+    using u64 = unsigned long long;
+    constexpr int L = kAdjL, RC = kAdjRC, NS = kAdjNS, BIN = S::BIN;
+    extern __shared__ __align__(128) unsigned char smem[];
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + S::BAR_OFF);     // [NS] chunk landed
+    uint64_t* empty = full + NS;                                          // [NS] every consumer warp is done with it
+    volatile int* sdead = reinterpret_cast<volatile int*>(full + 2 * NS);
+    float* ghs = reinterpret_cast<float*>(smem + S::GH_OFF);              // [T][NCT]
+
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int c0 = blockIdx.y * NCT;
+    const int T = a.T;
+    const long long n_raw = a.n_spectra + T - 1;
     const long long tiles = (n_raw + L - 1) / L;
-    const float2* taps2 = reinterpret_cast<const float2*>(a.taps);   // [t][pair]
-    for (long long u = blockIdx.x; u < tiles * a.n_streams; u += gridDim.x) {
-        const long long strm = u / tiles, r0 = (u - strm * tiles) * L;
-        const float2* g = a.gy + (size_t)strm * S * C;
-        // tap t (>= 1) brings row r0 - t (zero outside the stream) and h[t]
-        // into staging slot (t - 1) mod D, requested D taps ahead
-        auto stage = [&](int t) {
-            if (t < T) {
-                const int slot = (t - 1) % D;
-                const long long r = r0 - t;
-                if (r >= 0 && r < S) cp_async<16>(&sg[slot][tl], g + (size_t)r * C + 2 * p);
-                else sg[slot][tl] = make_float4(0.f, 0.f, 0.f, 0.f);
-                cp_async<8>(&sh[slot][tl], taps2 + (size_t)t * (C / 2) + p);
-            }
-            cp_async_commit();
-        };
-#pragma unroll
-        for (int d = 1; d <= D; ++d) stage(d);
-        // slot m mod L holds g_y row r0 + m; at tap t output j reads row r0 + j - t
-        unsigned long long wr[L], wi[L], ar[L], ai[L];
-#pragma unroll
-        for (int j = 0; j < L; ++j) {
-            const long long r = r0 + j;
-            load_gpair(g + (size_t)r * C, p, r < S, wr[j], wi[j]);
-            ar[j] = ai[j] = 0ull;
+    const int nch = L / RC + (T + RC - 1) / RC;
+    if (tid == 0) {
+        for (int i = 0; i < NS; ++i) {
+            mbar_init(&full[i], 1);
+            mbar_init(&empty[i], NCT / 32);
         }
-        unsigned long long hh;
-        {
-            const float2 h = __ldg(taps2 + p);
-            hh = pk2(h.x, h.y);
-        }
-        for (int tb = 0; tb < T; tb += L) {
-#pragma unroll
-            for (int v = 0; v < L; ++v) {
-                const int t = tb + v;
-                if (t < T) {
-                    if (t > 0) {                                 // row r0 - t enters slot (-t) mod L
-                        const int slot = (v + L - 1) % D;        // (t - 1) mod D
-                        cp_async_wait<D - 1>();
-                        const float4 gv = sg[slot][tl];
-                        wr[(L - v) % L] = pk2(gv.x, gv.z);
-                        wi[(L - v) % L] = pk2(gv.y, gv.w);
-                        const float2 h = sh[slot][tl];
-                        hh = pk2(h.x, h.y);
-                        stage(t + D);
-                    }
-#pragma unroll
-                    for (int j = 0; j < L; ++j) {
-                        ffma2(ar[j], hh, wr[(j - v + L) % L]);
-                        ffma2(ai[j], hh, wi[(j - v + L) % L]);
-                    }
-                }
-            }
-        }
-        cp_async_wait<0>();
-        float4* out = reinterpret_cast<float4*>(a.gx + (size_t)strm * a.gx_stride);
-#pragma unroll
-        for (int j = 0; j < L; ++j) {
-            const long long r = r0 + j;
-            if (r < n_raw) {
-                const float2 re = upk2(ar[j]), im = upk2(ai[j]);
-                out[(size_t)r * (C / 2) + p] = make_float4(re.x, im.x, re.y, im.y);
-            }
-        }
+        fence_mbar_init();
+        *sdead = 0;
     }
-}
+    if (GH && tid < NCT)
+        for (int t = 0; t < T; ++t) ghs[t * NCT + tid] = 0.f;
+    __syncthreads();
 
-struct AdjCorrArgs {
-    const float2* gy;        // g_y, n_spectra*C per stream, streams contiguous
-    const void* x;           // forward input (plan's type), n_raw*C per stream, streams x_stride apart
-    float* partials;         // n_parts rows of TM*C partial sums
-    long long n_spectra, n_streams, x_stride;
-    int C, T, TM, n_parts;
-};
-
-
-// grid.x: parts of the rows of all streams, grid.y: blocks of channel pairs,
-// grid.z: blocks of kAdjTB taps.  Each thread streams its rows through kAdjStage
-// shared-memory staging slots of its own (cp.async), so kAdjStage rows of g_y and x
-// are in flight while it works on the oldest.
-template <int IN>
-__global__ void __launch_bounds__(128, 4) pfb_bwd_gradh_kernel(AdjCorrArgs a) {
-    constexpr int TB = kAdjTB, BIN = InTraits<IN>::bytes, XB = 2 * BIN, D = kAdjStage;
-    static_assert(TB % D == 0 || D % TB == 0, "staging slots and window slots repeat together");
-    __shared__ __align__(16) float4 sg[D][128];                      // g_y pair of a staged row
-    __shared__ __align__(16) unsigned char sx[D][128 * XB];          // x pair of a staged row
-    const int C = a.C, T = a.T;
-    const int tl = threadIdx.x;
-    const int p = blockIdx.y * blockDim.x + tl;                      // channel pair
-    const bool active = p < C / 2;
-    const int t0 = blockIdx.z * TB;
-    const long long S = a.n_spectra, n_raw = S + T - 1;
-    const long long R = S * a.n_streams;
-    long long u = (long long)blockIdx.x * R / a.n_parts;
-    const long long u1 = (long long)(blockIdx.x + 1) * R / a.n_parts;
-    unsigned long long acc[TB];
-#pragma unroll
-    for (int v = 0; v < TB; ++v) acc[v] = 0ull;
-    auto unpack_x = [&](const unsigned char* q, unsigned long long& re, unsigned long long& im) {
-        const float4 v = load_pair_smem<IN>(q);
-        re = pk2(v.x, v.z);
-        im = pk2(v.y, v.w);
+    BatchShare share(tiles, a.n_streams, blockIdx.x, gridDim.x);
+    long long strm, lo, hi;
+    // chunk use g sits in slot g mod NS and completes phase g / NS of its barriers
+    int slot = 0;
+    uint32_t phase = 0;
+    auto advance = [&] {
+        if (++slot == NS) {
+            slot = 0;
+            phase ^= 1;
+        }
     };
-    while (active && u < u1) {                                        // segments of single streams
-        const long long strm = u / S, s0 = u - strm * S;
-        const long long s1 = (u1 - strm * S < S) ? u1 - strm * S : S;
-        u = strm * S + s1;
-        const float2* g = a.gy + (size_t)strm * S * C;
-        const unsigned char* x = static_cast<const unsigned char*>(a.x) + (size_t)strm * a.x_stride * BIN;
-        // stage row s: g_y row s and the x row entering the window there, s + t0 + TB - 1
-        auto stage = [&](long long s, int slot) {
-            if (s < s1) {
-                cp_async<16>(&sg[slot][tl], g + (size_t)s * C + 2 * p);
-                const long long r = s + t0 + TB - 1;
-                if (r < n_raw) {
-                    cp_async<XB>(&sx[slot][tl * XB], x + ((size_t)r * C + 2 * p) * BIN);
-                } else {
-                    float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-                    memcpy(&sx[slot][tl * XB], &z, XB);
+    if (tid >= NCT) {
+        // ------------------------------------------------ producer warp
+        long long issued = 0;
+        bool ok = true;
+        while (ok && share.next(strm, lo, hi)) {
+            for (long long k = lo; ok && k < hi; ++k) {
+                for (int c = 0; c < nch; ++c) {
+                    if (issued >= NS) ok = !*sdead && mbar_wait_bounded(&empty[slot], phase ^ 1, kWaitLimitNs);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    if (lane == 0) {
+                        unsigned char* dst = smem + slot * S::CHUNKB;
+                        fence_proxy_async_smem();
+                        const int u = (c - L / RC) * RC;             // the chunk's first step
+                        const bool first = u < 0;
+                        mbar_expect_tx(&full[slot], S::GB + (first ? (GH ? RC * NCT * BIN : 0) : RC * NCT * 4));
+                        tma_load_box3(dst, &g_map, c0, (int)(k * L) - (T - 1) + c * RC, (int)strm, &full[slot]);
+                        if (!first) tma_load_box2(dst + S::GB, &tap_map, c0, T - RC - u, &full[slot]);
+                        else if (GH) tma_load_box3(dst + S::GB, &x_map, c0, (int)(k * L) + c * RC, (int)strm, &full[slot]);
+                    }
+                    __syncwarp();
+                    ++issued;
+                    advance();
                 }
             }
-            cp_async_commit();
-        };
-        // slot m mod TB holds x row s0 + t0 + m (re pair, im pair); at row s0 + i,
-        // tap t0 + v reads row s0 + i + t0 + v, slot (i + v) mod TB
-        unsigned long long xr[TB], xi[TB];
-#pragma unroll
-        for (int m = 0; m + 1 < TB; ++m) {
-            const long long r = s0 + t0 + m;
-            const float4 v = r < n_raw ? load_pair_global<IN>(x, r * C + 2 * p) : make_float4(0.f, 0.f, 0.f, 0.f);
-            xr[m] = pk2(v.x, v.z);
-            xi[m] = pk2(v.y, v.w);
         }
+        if (!ok && lane == 0 && !*sdead) {
+            atomicExch(a.err, 1);
+            *sdead = 1;
+        }
+        // leave only after every copy of this CTA has landed
+        for (long long i = 0; i < NS && i < issued; ++i) {
+            if (slot == 0) {
+                slot = NS;
+                phase ^= 1;
+            }
+            --slot;
+            mbar_wait_bounded(&full[slot], phase, kWaitLimitNs);
+        }
+        return;
+    }
+
+    // ---------------------------------------------------- consumer warps
+    auto wait_full = [&] {
+        if (mbar_try_wait(&full[slot], phase) || *sdead) return;
+        if (!mbar_wait_bounded(&full[slot], phase, kWaitLimitNs)) {
+            atomicExch(a.err, 1);
+            *sdead = 1;
+        }
+    };
+    auto release = [&] {
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cta(&empty[slot]);
+        advance();
+    };
+    while (share.next(strm, lo, hi)) {
+        for (long long k = lo; k < hi; ++k) {
+            const long long r0 = k * L;
+            u64 acc[GX ? L : 1], win[L], xs[GH ? L : 1];
+            if constexpr (GX) {
 #pragma unroll
-        for (int d = 0; d < D; ++d) stage(s0 + d, d);
-        for (long long ib = 0; ib < s1 - s0; ib += TB) {
+                for (int j = 0; j < L; ++j) acc[j] = 0ull;
+            }
+            auto load_g = [&](int i, u64& w) {
+                w = *reinterpret_cast<const u64*>(smem + slot * S::CHUNKB + (i * NCT + tid) * 8);
+            };
 #pragma unroll
-            for (int i = 0; i < TB; ++i) {
-                const long long s = s0 + ib + i;
-                if (s < s1) {
-                    const int slot = i % D;                           // (s - s0) mod D
-                    cp_async_wait<D - 1>();                           // row s has landed
-                    const float4 gv = sg[slot][tl];
-                    const unsigned long long gr = pk2(gv.x, gv.z), gi = pk2(gv.y, gv.w);
-                    unpack_x(&sx[slot][tl * XB], xr[(i + TB - 1) % TB], xi[(i + TB - 1) % TB]);
-                    stage(s + D, slot);
+            for (int c = 0; c < L / RC; ++c) {
+                wait_full();
 #pragma unroll
-                    for (int v = 0; v < TB; ++v) {
-                        ffma2(acc[v], gr, xr[(i + v) % TB]);
-                        ffma2(acc[v], gi, xi[(i + v) % TB]);
+                for (int i = 0; i < RC; ++i) {
+                    load_g(i, win[c * RC + i]);
+                    if constexpr (GH) {
+                        const float2 v = load_one_smem<IN>(smem + slot * S::CHUNKB + S::GB + (i * NCT + tid) * BIN);
+                        xs[c * RC + i] = pk2(v.x, v.y);
                     }
                 }
+                release();
+            }
+            auto steps = [&](auto edge_tag) {
+                // EDGE (FP32 input): some rows lie outside the stream; their zeros must
+                // not meet an inf or NaN sample
+                constexpr bool EDGE = decltype(edge_tag)::value != 0;
+#pragma unroll 1
+                for (int tb = 0; tb < T; tb += L) {
+#pragma unroll
+                    for (int blk = 0; blk < L / RC; ++blk) {
+                        const int u0 = tb + blk * RC;
+                        if (u0 >= T) break;
+                        wait_full();
+#pragma unroll
+                        for (int i = 0; i < RC; ++i) {
+                            const int w = blk * RC + i;              // window slot of the oldest row
+                            const int t = T - 1 - u0 - i;
+                            if (t < 0) break;
+                            if constexpr (GX) {
+                                const float hv = *reinterpret_cast<const float*>(smem + slot * S::CHUNKB + S::GB +
+                                                                                 ((RC - 1 - i) * NCT + tid) * 4);
+                                const u64 h = pk2(hv, hv);
+#pragma unroll
+                                for (int j = 0; j < L; ++j) ffma2(acc[j], h, win[(j + w) % L]);
+                            }
+                            if constexpr (GH) {
+                                u64 p0 = 0ull, p1 = 0ull;
+#pragma unroll
+                                for (int j = 0; j < L; ++j) {
+                                    u64 x = xs[j];
+                                    if constexpr (EDGE) {
+                                        const long long s = r0 + j - t;
+                                        if (s < 0 || s >= a.n_spectra) x = 0ull;
+                                    }
+                                    ffma2(j & 1 ? p1 : p0, win[(j + w) % L], x);
+                                }
+                                const float2 p = upk2(add2(p0, p1));
+                                ghs[t * NCT + tid] += p.x + p.y;
+                            }
+                            load_g(i, win[w]);
+                        }
+                        release();
+                    }
+                }
+            };
+            if (GH && IN == IN_CF32 && (r0 < T - 1 || r0 + L > a.n_spectra)) steps(ic<1>{});
+            else steps(ic<0>{});
+            if constexpr (GX) {
+                if (!*sdead) {
+                    float2* out = a.gx + ((size_t)strm * n_raw + r0) * a.C + c0 + tid;
+#pragma unroll
+                    for (int j = 0; j < L; ++j)
+                        if (r0 + j < n_raw) __stcs(out + (size_t)j * a.C, upk2(acc[j]));
+                }
             }
         }
-        cp_async_wait<0>();
     }
-    if (!active) return;
-    float* part = a.partials + (size_t)blockIdx.x * a.TM * C;
-#pragma unroll
-    for (int v = 0; v < TB; ++v) {
-        const int t = t0 + v;
-        if (t < T) {
-            const float2 s = upk2(acc[v]);
-            *reinterpret_cast<float2*>(part + (size_t)t * C + 2 * p) = s;
-        }
+    if constexpr (GH) {
+        float* part = a.partials + (size_t)blockIdx.x * a.TM * a.C + c0 + tid;
+        for (int t = 0; t < T; ++t) part[(size_t)t * a.C] = ghs[t * NCT + tid];
     }
 }
 

@@ -35,9 +35,8 @@
 // (spills: 116), refills by the last warp off a slot (73).
 #pragma once
 
-#include <cuda.h>
-
 #include "ppf_fwd_carry.cuh"
+#include "ppf_tmap.h"
 
 namespace ppf {
 
@@ -256,31 +255,10 @@ pfb_fwd_longtap_kernel(FwdArgs args, const __grid_constant__ CUtensorMap in_map,
 // Tensor maps of a launch: the streams' samples as (channel, row, stream) in
 // boxes of 8 rows of NCT channels, and the plan's tap table (64 rows).
 inline cudaError_t longtap_maps(const FwdArgs& a, int C, int bin, int nct, CUtensorMap* in_map, CUtensorMap* tap_map) {
-    using Encode = decltype(&cuTensorMapEncodeTiled);
-    static const Encode encode = [] {
-        void* fn = nullptr;
-        cudaDriverEntryPointQueryResult found;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found) != cudaSuccess ||
-            found != cudaDriverEntryPointSuccess)
-            fn = nullptr;
-        return reinterpret_cast<Encode>(fn);
-    }();
-    if (encode == nullptr) return cudaErrorNotSupported;
-    const cuuint64_t n_raw = (cuuint64_t)(a.n_spectra + a.T - 1);
-    const cuuint64_t stride = a.n_streams > 1 ? (cuuint64_t)a.in_stride * bin : n_raw * C * bin;
-    const cuuint64_t dims[3] = {(cuuint64_t)C, n_raw, (cuuint64_t)a.n_streams}, strides[2] = {(cuuint64_t)C * bin, stride};
-    const cuuint32_t box[3] = {(cuuint32_t)nct, 8, 1}, one[3] = {1, 1, 1};
-    const CUtensorMapDataType type = bin == 2 ? CU_TENSOR_MAP_DATA_TYPE_UINT16
-                                   : bin == 4 ? CU_TENSOR_MAP_DATA_TYPE_UINT32 : CU_TENSOR_MAP_DATA_TYPE_INT64;
-    if (encode(in_map, type, 3, const_cast<void*>(a.in), dims, strides, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
-               CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return cudaErrorInvalidValue;
-    const cuuint64_t tdims[2] = {(cuuint64_t)C, 64}, tstride[1] = {(cuuint64_t)C * 4};
-    if (encode(tap_map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(a.taps), tdims, tstride, box, one,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return cudaErrorInvalidValue;
-    return cudaSuccess;
+    const unsigned long long n_raw = a.n_spectra + a.T - 1, row = (unsigned long long)C * bin;
+    const cudaError_t ce = make_tmap(in_map, a.in, bin, C, n_raw, row, a.n_streams,
+                                     a.n_streams > 1 ? a.in_stride * bin : n_raw * row, nct, 8);
+    return ce != cudaSuccess ? ce : make_tmap(tap_map, a.taps, 4, C, 64, C * 4ull, 0, 0, nct, 8);
 }
 
 template <int C, int IN, int OUT, int DIV>

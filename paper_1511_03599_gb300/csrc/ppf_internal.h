@@ -16,8 +16,7 @@ ppf_status set_error(ppf_status s, const char* fmt, ...);
 struct FwdArgs;
 struct BwdArgs;
 struct IdftArgs;
-struct AdjFirArgs;
-struct AdjCorrArgs;
+struct AdjArgs;
 
 struct FwdEntry {
     int threads;     // threads per CTA
@@ -65,12 +64,11 @@ struct IdftEntry {
     const void* fn;
     cudaError_t (*launch)(const IdftArgs&, int grid, cudaStream_t);
 };
-// grad_x pass; grid_x: CTAs along the row tiles of all streams.
-cudaError_t bwd_gradx(const AdjFirArgs& a, int grid_x, cudaStream_t st);
-// grad_h partial sums (a.n_parts parts of the rows of all streams).
-cudaError_t bwd_gradh(int in, const AdjCorrArgs& a, cudaStream_t st);
-// Tap blocks of the grad_h pass (partial-sum rows are TM*C floats).
-int bwd_gradh_tap_blocks(int T);
+// Parts of the row tiles that fill the GPU once, and the pass itself (a.gx or
+// a.partials may be null: that sum is not wanted).
+int bwd_grad_parts(int in, int C, int T, int sms, long long n_raw, long long n_streams);
+cudaError_t bwd_grad(int in, const AdjArgs& a, const float2* gy, const void* x, const float* taps, int parts,
+                     cudaStream_t st);
 
 // Per-C lookups; return false when the (tap bucket, in, out) triple is not built.
 #define PPF_DECLARE_C(C)                                                         \
