@@ -96,7 +96,7 @@ bool lookup_fir(int C, int tm, int in, ppf::FwdEntry* e) {
     }
 }
 
-bool lookup_idft(int C, ppf::IdftEntry* e) {
+bool lookup_idft(int C, ppf::FwdEntry* e) {
     switch (C) {
 #define PPF_ID(CC) case CC: return ppf::idft_lookup_c##CC(e);
         PPF_ID(32) PPF_ID(64) PPF_ID(128) PPF_ID(256) PPF_ID(512) PPF_ID(1024) PPF_ID(2048) PPF_ID(4096)
@@ -115,6 +115,15 @@ bool twiddles(int C, std::vector<float>& pairs) {
 #undef PPF_TW
         default: return false;
     }
+}
+
+// Let every kernel of an entry use its dynamic shared memory.
+cudaError_t allow_smem(const ppf::FwdEntry& e) {
+    const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaError_t ce = cudaFuncSetAttribute(e.fn, attr, e.smem);
+    if (ce == cudaSuccess && e.small_batch > 0) ce = cudaFuncSetAttribute(e.small_fn, attr, e.small_smem);
+    if (ce == cudaSuccess && e.short_fn != nullptr) ce = cudaFuncSetAttribute(e.short_fn, attr, e.smem);
+    return ce;
 }
 
 int bytes_in(ppf_in_t t) { return t == PPF_IN_CI8 ? 2 : t == PPF_IN_CI16 ? 4 : 8; }
@@ -156,8 +165,9 @@ struct ppf_plan_s {
     int bwd_occupancy;
     float* d_partials;    // tap-gradient partial sums, one row of TM*C per CTA (or per part)
     long long partials_ctas;
-    ppf::IdftEntry idft;  // unfused adjoint: inverse DFT pass
-    int idft_occupancy;
+    ppf::FwdEntry idft;   // unfused adjoint: inverse DFT pass
+    int idft_grid;
+    float* d_ones;        // its C unit taps (behind the twiddles)
     float2* d_gy;         // unfused adjoint: g_y scratch
     size_t gy_bytes;
     bool has_fir;         // FIR-only ablation kernel available for this shape
@@ -227,16 +237,8 @@ extern "C" ppf_status ppf_plan(ppf_plan_t* out, int C, int T, const float* coeff
     int sms = 0;
     ce = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (ce != cudaSuccess) return cuda_fail(ce, "ppf_plan: SM count");
-    ce = cudaFuncSetAttribute(e.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, e.smem);
+    ce = allow_smem(e);
     if (ce != cudaSuccess) return cuda_fail(ce, "ppf_plan: shared memory attribute");
-    if (e.small_batch > 0) {
-        ce = cudaFuncSetAttribute(e.small_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, e.small_smem);
-        if (ce != cudaSuccess) return cuda_fail(ce, "ppf_plan: shared memory attribute");
-    }
-    if (e.short_fn != nullptr) {
-        ce = cudaFuncSetAttribute(e.short_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, e.smem);
-        if (ce != cudaSuccess) return cuda_fail(ce, "ppf_plan: shared memory attribute");
-    }
     int occ = 0, grid_ctas = 0;
     if (e.cluster > 0) {
         // persistent grid: as many whole clusters as can be resident at once
@@ -258,6 +260,8 @@ extern "C" ppf_status ppf_plan(ppf_plan_t* out, int C, int T, const float* coeff
     std::memcpy(taps.data(), coeffs_host, sizeof(float) * (size_t)C * T);
     std::vector<float> tw;
     twiddles(C, tw);
+    const size_t ones_at = tw.size();
+    tw.resize(ones_at + C, 1.f);
 
     ppf_plan_s* p = new (std::nothrow) ppf_plan_s{};
     if (p == nullptr) return fail(PPF_ERR_OUT_OF_MEMORY, "ppf_plan: host allocation");
@@ -276,14 +280,15 @@ extern "C" ppf_status ppf_plan(ppf_plan_t* out, int C, int T, const float* coeff
         p->has_bwd = p->bwd_occupancy > 0;
     }
     if (lookup_idft(C, &p->idft)) {
-        ce = cudaFuncSetAttribute(p->idft.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, p->idft.smem);
+        int iocc = 0;
+        ce = allow_smem(p->idft);
         if (ce == cudaSuccess)
-            ce = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p->idft_occupancy, p->idft.fn, p->idft.threads,
-                                                               p->idft.smem);
+            ce = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&iocc, p->idft.fn, p->idft.threads, p->idft.smem);
         if (ce != cudaSuccess) {
             delete p;
             return cuda_fail(ce, "ppf_plan: inverse-DFT kernel attributes");
         }
+        p->idft_grid = sms * iocc;
     }
     if (lookup_fir(C, tm, (int)in_dtype, &p->fir)) {
         int focc = 0;
@@ -308,6 +313,7 @@ extern "C" ppf_status ppf_plan(ppf_plan_t* out, int C, int T, const float* coeff
         ppf_destroy(p);
         return s;
     }
+    p->d_ones = reinterpret_cast<float*>(p->d_tw) + ones_at;
     *out = p;
     return PPF_OK;
 }
@@ -335,6 +341,34 @@ static long long work_units(long long resident, long long n_streams, long long b
     return std::max<long long>(1, std::min<long long>(resident, total));
 }
 
+// Launch one of an entry's kernels: `resident` CTAs of e.fn fit the device at once.
+static ppf_status launch_entry(const ppf::FwdEntry& e, int resident, int sms, const ppf::FwdArgs& a, const char* what,
+                               cudaStream_t st) {
+    const long long n = a.n_spectra, n_streams = a.n_streams;
+    const long long nb = (n + e.batch - 1) / e.batch;
+    const int unit = e.cluster > 0 ? e.cluster : 1;                // CTAs per work unit
+    auto* launch = e.launch;
+    long long grid;
+    // a call that gives each SM at most one small batch runs on those
+    const long long n_small = e.small_batch > 0 && n <= sms * (long long)e.small_batch
+                                  ? n_streams * ((n + e.small_batch - 1) / e.small_batch) : sms + 1ll;
+    if (n_small <= sms) {
+        grid = n_small;
+        launch = e.small_launch;
+    } else if ((e.variant & 4) && e.cluster == 0) {
+        // carry kernel: the same number of CTAs on every stream, one wave if
+        // the streams allow it (at least one CTA, at most one per batch)
+        const long long cps = std::max<long long>(1, std::min<long long>(resident / n_streams, nb));
+        grid = cps * n_streams;
+        if (grid > 0x7fffffffll) return fail(PPF_ERR_INVALID_ARG, "%s: too many streams", what);
+        if (nb <= cps * ppf::kCarryShort && e.short_launch != nullptr) launch = e.short_launch;
+    } else {
+        grid = work_units(resident / unit, n_streams, nb) * unit;
+    }
+    const cudaError_t ce = launch(a, (int)grid, st);
+    return ce == cudaSuccess ? PPF_OK : cuda_fail(ce, what);
+}
+
 static ppf_status launch_fwd(ppf_plan_t p, const void* in_dev, long long in_stride, void* out_dev,
                              long long out_stride, long long n, long long n_streams, cudaStream_t st) {
     ppf::FwdArgs a;
@@ -348,36 +382,8 @@ static ppf_status launch_fwd(ppf_plan_t p, const void* in_dev, long long in_stri
     a.n_spectra = n;
     a.T = p->T;
     a.flags = p->debug_flags;
-    const long long nb = (n + p->fwd.batch - 1) / p->fwd.batch;
-    const int unit = p->fwd.cluster > 0 ? p->fwd.cluster : 1;      // CTAs per work unit
     a.n_streams = n_streams;
-    long long grid;
-    // a call that gives each SM at most one small batch runs on those
-    const long long n_small =
-        p->fwd.small_batch > 0 && n <= p->sms * (long long)p->fwd.small_batch
-            ? n_streams * ((n + p->fwd.small_batch - 1) / p->fwd.small_batch) : p->sms + 1ll;
-    if (n_small <= p->sms) {
-        cudaError_t ce = p->fwd.small_launch(a, (int)n_small, st);
-        if (ce != cudaSuccess) return cuda_fail(ce, "ppf_execute: launch");
-        return PPF_OK;
-    }
-    if ((p->fwd.variant & 4) && p->fwd.cluster == 0) {
-        // carry kernel: the same number of CTAs on every stream, one wave if
-        // the streams allow it (at least one CTA, at most one per batch)
-        const long long cps = std::max<long long>(1, std::min<long long>(p->grid / n_streams, nb));
-        grid = cps * n_streams;
-        if (grid > 0x7fffffffll) return fail(PPF_ERR_INVALID_ARG, "ppf_execute: too many streams");
-        if (nb <= cps * ppf::kCarryShort && p->fwd.short_launch != nullptr) {
-            cudaError_t ce = p->fwd.short_launch(a, (int)grid, st);
-            if (ce != cudaSuccess) return cuda_fail(ce, "ppf_execute: launch");
-            return PPF_OK;
-        }
-    } else {
-        grid = work_units(p->grid / unit, n_streams, nb) * unit;
-    }
-    cudaError_t ce = p->fwd.launch(a, (int)grid, st);
-    if (ce != cudaSuccess) return cuda_fail(ce, "ppf_execute: launch");
-    return PPF_OK;
+    return launch_entry(p->fwd, p->grid, p->sms, a, "ppf_execute: launch", st);
 }
 
 static bool overlaps(const void* a, unsigned long long na, const void* b, unsigned long long nb) {
@@ -418,7 +424,7 @@ extern "C" ppf_status ppf_execute(ppf_plan_t p, const void* in_dev, void* out_de
 static ppf_status backward_unfused(ppf_plan_t p, const void* grad_out_dev, const void* in_dev, void* grad_in_dev,
                                    float* grad_taps_dev, long long n_spectra, long long n_streams, cudaStream_t st) {
     const int C = p->C, T = p->T, TM = p->TM;
-    if (p->idft.fn == nullptr || p->idft_occupancy < 1)
+    if (p->idft.fn == nullptr || p->idft_grid < 1)
         return fail(PPF_ERR_UNSUPPORTED, "ppf_backward: no inverse-DFT kernel for C=%d", C);
     const long long n_raw = n_spectra + T - 1;
     const size_t gy_bytes = (size_t)n_streams * n_spectra * C * 8;
@@ -431,17 +437,19 @@ static ppf_status backward_unfused(ppf_plan_t p, const void* grad_out_dev, const
         if (ce != cudaSuccess) return cuda_fail(ce, "ppf_backward: g_y scratch");
         p->gy_bytes = gy_bytes;
     }
-    ppf::IdftArgs ia;
-    ia.gY = static_cast<const float2*>(grad_out_dev);
-    ia.gy = p->d_gy;
+    ppf::FwdArgs ia;
+    ia.in = grad_out_dev;
+    ia.out = p->d_gy;
+    ia.in_stride = ia.out_stride = n_spectra * C;
+    ia.taps = p->d_ones;
     ia.tw = p->d_tw;
+    ia.err = p->d_err;
     ia.n_spectra = n_spectra;
-    ia.gY_stride = n_spectra * C;
     ia.n_streams = n_streams;
-    const long long idft_grid = work_units((long long)p->sms * p->idft_occupancy, n_streams,
-                                           (n_spectra + p->idft.batch - 1) / p->idft.batch);
-    ce = p->idft.launch(ia, (int)idft_grid, st);
-    if (ce != cudaSuccess) return cuda_fail(ce, "ppf_backward: inverse DFT launch");
+    ia.T = 1;
+    ia.flags = 0;
+    const ppf_status is = launch_entry(p->idft, p->idft_grid, p->sms, ia, "ppf_backward: inverse DFT launch", st);
+    if (is != PPF_OK) return is;
     // parts of the row tiles of all streams, one CTA per part and channel block;
     // partial sums capped at 2^25 floats
     long long parts = ppf::bwd_grad_parts((int)p->in, C, T, p->sms, n_raw, n_streams);

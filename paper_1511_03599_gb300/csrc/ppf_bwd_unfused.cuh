@@ -9,9 +9,10 @@
 //   grad_x[r][c] = sum_{t<T} h[t][c] g_y[r-t][c]  (transposed FIR, Alg. 1)
 //   grad_h[t][c] = sum_s Re(conj(g_y[s][c]) x[s+t][c])
 // (g_y[s] = 0 outside 0 <= s < S) run as separate kernels:
-//   1. pfb_bwd_idft_kernel<C>: batches of G rows through shared memory, the
-//      forward's DFT stages in their inverse mode (conj(F conj(.))), g_y rows
-//      to the scratch;
+//   1. the forward kernels with one unit tap and conjugated input and output
+//      (conj(F conj(.))) on the rows of G, g_y rows to the scratch (C = 512, 65536
+//      rows: 85 us; 120 with a kernel of its own that copied rows in and out
+//      between CTA-wide stages);
 //   2. pfb_bwd_grad_kernel<IN>: both other sums from one pass over g_y, one
 //      thread per channel, a window of kAdjL rows of g_y in registers, rows,
 //      samples and taps through a TMA ring; per-part partial sums of grad_h
@@ -25,26 +26,19 @@
 
 namespace ppf {
 
-struct IdftArgs {
-    const float2* gY;        // incoming gradient, n_spectra*C per stream, streams gY_stride apart
-    float2* gy;              // g_y, n_spectra*C per stream, streams contiguous
-    const float2* tw;        // the forward plan's twiddle tables
-    long long n_spectra, gY_stride, n_streams;
-};
-
-// Threads and batch of the forward's generic kernel in its plain
-// configuration (for these its DFT stages divide their items exactly):
-// 64 KB of spectra per batch (48 KB for C = 384/768/1536, 96 KB at 3072).
+// Pass 1 at C = 32, where no forward kernel conjugates: 256 rows of G at a time
+// through shared memory, the DFT stages in their inverse mode.  args.in: G,
+// args.out: g_y (n_spectra*C per stream, strides as for the forward).
 template <int C>
 struct IdftShape {
-    static constexpr int NT = C >= 2048 ? 512 : 256;
-    static constexpr int B = C >= 4096 ? 2 : C >= 2048 ? 4 : is_c3(C) ? 16 * 384 / C : 8192 / C;
+    static constexpr int NT = 256;
+    static constexpr int B = 8192 / C;
     static constexpr int YBYTES = B * C * 8;
     static constexpr int SMEM = YBYTES + tw_size(C) * 8;
 };
 
 template <int C>
-__global__ void __launch_bounds__(IdftShape<C>::NT) pfb_bwd_idft_kernel(IdftArgs a) {
+__global__ void __launch_bounds__(IdftShape<C>::NT) pfb_bwd_idft_kernel(FwdArgs a) {
     using S = IdftShape<C>;
     constexpr int NT = S::NT, B = S::B, NST = fft_stages(C);
     extern __shared__ __align__(128) unsigned char smem[];
@@ -56,8 +50,8 @@ __global__ void __launch_bounds__(IdftShape<C>::NT) pfb_bwd_idft_kernel(IdftArgs
     BatchShare share((a.n_spectra + B - 1) / B, a.n_streams, blockIdx.x, gridDim.x);
     long long strm, lo, hi;
     while (share.next(strm, lo, hi)) {
-        const float4* src = reinterpret_cast<const float4*>(a.gY + (size_t)strm * a.gY_stride);
-        float4* dst = reinterpret_cast<float4*>(a.gy + (size_t)strm * a.n_spectra * C);
+        const float4* src = reinterpret_cast<const float4*>(static_cast<const float2*>(a.in) + (size_t)strm * a.in_stride);
+        float4* dst = reinterpret_cast<float4*>(static_cast<float2*>(a.out) + (size_t)strm * a.out_stride);
         for (long long k = lo; k < hi; ++k) {
             const long long s0 = k * B;
             const int rows = (int)(a.n_spectra - s0 < B ? a.n_spectra - s0 : B);
@@ -303,23 +297,6 @@ pfb_bwd_grad_kernel(AdjArgs a, const __grid_constant__ CUtensorMap g_map, const 
         float* part = a.partials + (size_t)blockIdx.x * a.TM * a.C + c0 + tid;
         for (int t = 0; t < T; ++t) part[(size_t)t * a.C] = ghs[t * NCT + tid];
     }
-}
-
-struct IdftInfo {
-    int threads, batch, smem;
-    const void* fn;
-};
-
-template <int C>
-inline IdftInfo idft_info() {
-    return IdftInfo{IdftShape<C>::NT, IdftShape<C>::B, IdftShape<C>::SMEM,
-                    reinterpret_cast<const void*>(&pfb_bwd_idft_kernel<C>)};
-}
-
-template <int C>
-inline cudaError_t idft_launch(const IdftArgs& a, int grid, cudaStream_t st) {
-    pfb_bwd_idft_kernel<C><<<grid, IdftShape<C>::NT, IdftShape<C>::SMEM, st>>>(a);
-    return cudaPeekAtLastError();
 }
 
 }  // namespace ppf

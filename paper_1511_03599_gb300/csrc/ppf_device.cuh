@@ -117,6 +117,8 @@ __device__ __forceinline__ float2 csub(float2 a, float2 b) {
 __device__ __forceinline__ float2 cmul(float2 a, float2 w) {
     return make_float2(fmaf(a.x, w.x, -a.y * w.y), fmaf(a.x, w.y, a.y * w.x));
 }
+template <bool CONJ>
+__device__ __forceinline__ float2 conj_if(float2 a) { return make_float2(a.x, CONJ ? -a.y : a.y); }
 // a * (-i)
 __device__ __forceinline__ float2 cmul_mi(float2 a) { return make_float2(a.y, -a.x); }
 

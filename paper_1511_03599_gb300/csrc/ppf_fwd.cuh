@@ -343,8 +343,10 @@ struct HalfGroup {
 // INV: the unnormalised inverse DFT (sign +i) computed as conj(DFT(conj(.)));
 // its last stage writes the result back into the spectrum's own row of
 // ybuf in natural order instead of to global memory.
+// CONJ: the last stage stores conjugates (the other half of an inverse DFT
+// whose caller conjugates the input).
 template <int C, int B, int NT, int P, int OUT, bool TW_SMEM, int SPW = 0, bool INV = false, bool SMEM_OUT = false,
-          int LAYOUT = 0, class GRP = CtaGroup, bool OOP = false>
+          int LAYOUT = 0, class GRP = CtaGroup, bool OOP = false, bool CONJ = false>
 __device__ __forceinline__ void fft_stage(float2* __restrict__ ybuf, const float2* __restrict__ tws,
                                           void* __restrict__ out, long long sb, long long vlo, long long vhi,
                                           float2* __restrict__ dbuf = nullptr) {
@@ -429,7 +431,7 @@ __device__ __forceinline__ void fft_stage(float2* __restrict__ ybuf, const float
             const long long s = sb + sp;
             if (s >= vlo && s < vhi) {
 #pragma unroll
-                for (int k = 0; k < R; ++k) store_out<OUT>(out, s * C + prefix + PP * k, v[it][k]);
+                for (int k = 0; k < R; ++k) store_out<OUT>(out, s * C + prefix + PP * k, conj_if<CONJ>(v[it][k]));
             }
         }
     }

@@ -141,7 +141,10 @@ struct CarryShape : CarryShapeSel<C, TM, IN>::type {};
 // ranges the shifted form measured 1-3 % slower (C = 512, int8 and int16); on
 // short ones it saves up to half the time (C = 256, T = 8, FP32, 4096 spectra,
 // two batches per CTA: 8.5 -> 6.1 us).
-template <int C, int TM, int IN, int OUT, bool FIRONLY, class GRP, bool MULTI, bool SHORT = false>
+//
+// CONJ (T = 1, FP32): the unnormalised inverse DFT of the input rows, as
+// conj(DFT(conj(.))) -- the first pass of the three-pass adjoint.
+template <int C, int TM, int IN, int OUT, bool FIRONLY, class GRP, bool MULTI, bool SHORT = false, bool CONJ = false>
 __device__ __forceinline__ bool carry_range(const FwdArgs& args, const void* in, void* out, long long lo, long long hi,
                                             unsigned char* smem) {
     using S = CarryShape<C, TM, IN>;
@@ -258,8 +261,9 @@ __device__ __forceinline__ bool carry_range(const FwdArgs& args, const void* in,
             float4 nxt[TM > 1 ? TM - 1 : 1];
 #pragma unroll
             for (int i = 0; i < B + TM - 1; ++i) {
-                const float4 x = (i < TM - 1) ? carry[i < TM - 1 ? i : 0]
-                                              : load_pair_smem<IN>(slot + (size_t)(i - (TM - 1)) * C * BIN);
+                float4 x = (i < TM - 1) ? carry[i < TM - 1 ? i : 0]
+                                        : load_pair_smem<IN>(slot + (size_t)(i - (TM - 1)) * C * BIN);
+                if constexpr (CONJ) x = make_float4(x.x, -x.y, x.z, -x.w);
                 const unsigned long long x01 = pk2(x.x, x.y), x23 = pk2(x.z, x.w);
 #pragma unroll
                 for (int j = 0; j < B; ++j) {
@@ -304,7 +308,7 @@ __device__ __forceinline__ bool carry_range(const FwdArgs& args, const void* in,
         if constexpr (!FIRONLY) {
             const long long sb = (lo + k) * B + sh - (T - 1);     // output spectrum of batch row 0
             static_for<NST>([&](auto p) {
-                fft_stage<C, B, NT, decltype(p)::value, OUT, S::TW_SMEM, S::SPW, false, false, S::LAYOUT, GRP>(
+                fft_stage<C, B, NT, decltype(p)::value, OUT, S::TW_SMEM, S::SPW, false, false, S::LAYOUT, GRP, false, CONJ>(
                     ybuf, tws, out, sb, vlo, vhi);
             });
         }
@@ -320,7 +324,7 @@ __device__ __forceinline__ bool carry_range(const FwdArgs& args, const void* in,
 // Most batches per CTA for the SHORT form.
 constexpr int kCarryShort = 16;
 
-template <int C, int TM, int IN, int OUT, bool FIRONLY = false, bool SHORT = false>
+template <int C, int TM, int IN, int OUT, bool FIRONLY = false, bool SHORT = false, bool CONJ = false>
 __global__ void __launch_bounds__(CarryShape<C, TM, IN>::NT, CarryShape<C, TM, IN>::MINB)
 pfb_fwd_carry_kernel(FwdArgs args) {
     using S = CarryShape<C, TM, IN>;
@@ -333,7 +337,7 @@ pfb_fwd_carry_kernel(FwdArgs args) {
     void* out = static_cast<unsigned char*>(args.out) + (size_t)strm * args.out_stride * (OUT == OUT_CF32 ? 8 : 4);
     const long long lo = (long long)bx * nbt / cps;
     const long long hi = (long long)(bx + 1) * nbt / cps;
-    carry_range<C, TM, IN, OUT, FIRONLY, CtaGroup, false, SHORT>(args, in, out, lo, hi, smem);
+    carry_range<C, TM, IN, OUT, FIRONLY, CtaGroup, false, SHORT, CONJ>(args, in, out, lo, hi, smem);
 }
 
 }  // namespace ppf

@@ -104,11 +104,60 @@ bool PPF_CAT(fir_lookup_c, PPF_C)(int tm, int in, FwdEntry* e) {
     }
 }
 
-bool PPF_CAT(idft_lookup_c, PPF_C)(IdftEntry* e) {
-    const IdftInfo i = idft_info<PPF_C>();
-    *e = IdftEntry{i.threads, i.batch, i.smem, i.fn, &idft_launch<PPF_C>};
-    return true;
+template <auto KERNEL, int NT, int SMEM>
+static cudaError_t launch_kernel(const FwdArgs& a, int grid, cudaStream_t st) {
+    KERNEL<<<grid, NT, SMEM, st>>>(a);
+    return cudaPeekAtLastError();
 }
+
+// The inverse DFT of the three-pass adjoint: the forward kernels with T = 1 and
+// conjugation; the small batches wherever the forward has them.
+template <int C>
+static bool make_idft(FwdEntry* e) {
+    *e = FwdEntry{};
+    e->tap_bucket = 1;
+    if constexpr (C == 32) {
+        using S = IdftShape<C>;
+        e->threads = S::NT;
+        e->batch = S::B;
+        e->smem = S::SMEM;
+        e->fn = reinterpret_cast<const void*>(&pfb_bwd_idft_kernel<C>);
+        e->launch = &launch_kernel<pfb_bwd_idft_kernel<C>, S::NT, S::SMEM>;
+        return true;
+    } else {
+        if constexpr (carry_preferred<C, 1, IN_CF32>()) {
+            using S = CarryShape<C, 1, IN_CF32>;
+            constexpr auto k = &pfb_fwd_carry_kernel<C, 1, IN_CF32, OUT_CF32, false, false, true>;
+            constexpr auto ks = &pfb_fwd_carry_kernel<C, 1, IN_CF32, OUT_CF32, false, true, true>;
+            e->threads = S::NT;
+            e->batch = S::B;
+            e->smem = S::SMEM;
+            e->variant = 4;
+            e->fn = reinterpret_cast<const void*>(k);
+            e->launch = &launch_kernel<k, S::NT, S::SMEM>;
+            e->short_fn = reinterpret_cast<const void*>(ks);
+            e->short_launch = &launch_kernel<ks, S::NT, S::SMEM>;
+        } else {
+            using S = RowShape<C, 1, IN_CF32>;
+            constexpr auto k = &pfb_fwd_row_kernel<C, 1, IN_CF32, OUT_CF32, 1, true>;
+            e->threads = S::NT;
+            e->batch = S::B;
+            e->smem = S::SMEM;
+            e->variant = 128;
+            e->fn = reinterpret_cast<const void*>(k);
+            e->launch = &launch_kernel<k, S::NT, S::SMEM>;
+        }
+        using M = RowShape<C, 1, IN_CF32, 4>;
+        constexpr auto km = &pfb_fwd_row_kernel<C, 1, IN_CF32, OUT_CF32, 4, true>;
+        e->small_batch = M::B;
+        e->small_smem = M::SMEM;
+        e->small_fn = reinterpret_cast<const void*>(km);
+        e->small_launch = &launch_kernel<km, M::NT, M::SMEM>;
+        return true;
+    }
+}
+
+bool PPF_CAT(idft_lookup_c, PPF_C)(FwdEntry* e) { return make_idft<PPF_C>(e); }
 
 int PPF_CAT(fwd_twiddle_count_c, PPF_C)() { return tw_total_float2s(PPF_C) > 0 ? tw_total_float2s(PPF_C) : 1; }
 

@@ -210,7 +210,8 @@ struct RowShape {
 // The row kernel's body over output batches [lo, hi) of one stream (in, out:
 // that stream's buffers), by a whole CTA of kRowThreads threads.  Returns
 // false when a bounded wait gave up.  Safe to call again for another range.
-template <int C, int TM, int IN, int OUT, int DIV = 1>
+// CONJ (T = 1, FP32): the unnormalised inverse DFT of the rows, conj(DFT(conj(.))).
+template <int C, int TM, int IN, int OUT, int DIV = 1, bool CONJ = false>
 __device__ __forceinline__ bool row_range(const FwdArgs& args, const void* in, void* out, long long lo, long long hi,
                                           unsigned char* smem) {
     using S = RowShape<C, TM, IN, DIV>;
@@ -349,10 +350,10 @@ __device__ __forceinline__ bool row_range(const FwdArgs& args, const void* in, v
                     if constexpr (PAIR) {
                         const float4 v = load_pair_smem<IN>(p);
                         x0 = pk2(v.x, v.z);
-                        x1 = pk2(v.y, v.w);
+                        x1 = CONJ ? pk2(-v.y, -v.w) : pk2(v.y, v.w);
                     } else {
                         const float2 v = load_one_smem<IN>(p);
-                        x0 = pk2(v.x, v.y);
+                        x0 = pk2(v.x, CONJ ? -v.y : v.y);
                     }
                 } else if constexpr (!S::STAGE) {
                     const long long r = row0 + seg + i;
@@ -360,10 +361,10 @@ __device__ __forceinline__ bool row_range(const FwdArgs& args, const void* in, v
                     if constexpr (PAIR) {
                         const float4 v = ok ? load_pair_global<IN>(in, r * C + a * M + col) : make_float4(0.f, 0.f, 0.f, 0.f);
                         x0 = pk2(v.x, v.z);
-                        x1 = pk2(v.y, v.w);
+                        x1 = CONJ ? pk2(-v.y, -v.w) : pk2(v.y, v.w);
                     } else {
                         const float2 v = ok ? load_one_global<IN>(in, r * C + a * M + col) : make_float2(0.f, 0.f);
-                        x0 = pk2(v.x, v.y);
+                        x0 = pk2(v.x, CONJ ? -v.y : v.y);
                     }
                 } else {
                     const int n = a * S::RW + i, gi = n / S::GR;
@@ -372,10 +373,10 @@ __device__ __forceinline__ bool row_range(const FwdArgs& args, const void* in, v
                     if constexpr (PAIR) {
                         const float4 v = load_pair_smem<IN>(p);
                         x0 = pk2(v.x, v.z);
-                        x1 = pk2(v.y, v.w);
+                        x1 = CONJ ? pk2(-v.y, -v.w) : pk2(v.y, v.w);
                     } else {
                         const float2 v = load_one_smem<IN>(p);
-                        x0 = pk2(v.x, v.y);
+                        x0 = pk2(v.x, CONJ ? -v.y : v.y);
                     }
                     if ((n % S::GR == S::GR - 1 || n + 1 == S::NROW) && gi + S::NCH < S::NGR) stage_group(k, gi + S::NCH);
                 }
@@ -565,7 +566,7 @@ __device__ __forceinline__ bool row_range(const FwdArgs& args, const void* in, v
                     float2* p = ybuf + (g * RPW + sl) * S::SS;
 #pragma unroll
                     for (int b = 0; b < RB; ++b) {
-                        if constexpr (OUT == OUT_CF32) p[e + SITEMS * b] = v[it][b];
+                        if constexpr (OUT == OUT_CF32) p[e + SITEMS * b] = conj_if<CONJ>(v[it][b]);
                         else reinterpret_cast<__half2*>(p)[e + SITEMS * b] = __float22half2_rn(v[it][b]);
                     }
                 }
@@ -592,7 +593,7 @@ __device__ __forceinline__ bool row_range(const FwdArgs& args, const void* in, v
                     const long long s = row0 + g * RPW + sl;
                     if (s < n_spectra) {
 #pragma unroll
-                        for (int b = 0; b < RB; ++b) store_out<OUT>(out, s * C + e + SITEMS * b, v[it][b]);
+                        for (int b = 0; b < RB; ++b) store_out<OUT>(out, s * C + e + SITEMS * b, conj_if<CONJ>(v[it][b]));
                     }
                 }
             }
@@ -613,7 +614,7 @@ __device__ __forceinline__ bool row_range(const FwdArgs& args, const void* in, v
     return true;
 }
 
-template <int C, int TM, int IN, int OUT, int DIV = 1>
+template <int C, int TM, int IN, int OUT, int DIV = 1, bool CONJ = false>
 __global__ void __launch_bounds__(kRowThreads, 1) pfb_fwd_row_kernel(FwdArgs args) {
     using S = RowShape<C, TM, IN, DIV>;
     extern __shared__ __align__(128) unsigned char smem[];
@@ -622,7 +623,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) pfb_fwd_row_kernel(FwdArgs arg
     while (share.next(strm, lo, hi)) {
         const void* in = static_cast<const unsigned char*>(args.in) + (size_t)strm * args.in_stride * S::BIN;
         void* out = static_cast<unsigned char*>(args.out) + (size_t)strm * args.out_stride * (OUT == OUT_CF32 ? 8 : 4);
-        if (!row_range<C, TM, IN, OUT, DIV>(args, in, out, lo, hi, smem)) return;
+        if (!row_range<C, TM, IN, OUT, DIV, CONJ>(args, in, out, lo, hi, smem)) return;
     }
 }
 

@@ -15,7 +15,6 @@ ppf_status set_error(ppf_status s, const char* fmt, ...);
 
 struct FwdArgs;
 struct BwdArgs;
-struct IdftArgs;
 struct AdjArgs;
 
 struct FwdEntry {
@@ -55,15 +54,8 @@ bool bwd_lookup(int C, int tap_bucket, int in, BwdEntry* e);
 cudaError_t bwd_reduce(const float* partials, int nparts, int T, int TM, int C, const int* err, float* grad_h,
                        cudaStream_t st);
 
-// Unfused adjoint (any planned shape): inverse DFT per C, then the
-// transposed FIR and the tap correlation (runtime C and T).
-struct IdftEntry {
-    int threads;     // threads per CTA
-    int batch;       // spectra per CTA batch
-    int smem;        // dynamic shared memory bytes
-    const void* fn;
-    cudaError_t (*launch)(const IdftArgs&, int grid, cudaStream_t);
-};
+// Unfused adjoint (any planned shape): inverse DFT per C (idft_lookup_c*, a
+// forward entry whose input is G and whose taps are ones), then both sums.
 // Parts of the row tiles that fill the GPU once, and the pass itself (a.gx or
 // a.partials may be null: that sum is not wanted).
 int bwd_grad_parts(int in, int C, int T, int sms, long long n_raw, long long n_streams);
@@ -74,7 +66,7 @@ cudaError_t bwd_grad(int in, const AdjArgs& a, const float2* gy, const void* x, 
 #define PPF_DECLARE_C(C)                                                         \
     bool fwd_lookup_c##C(int tap_bucket, int in, int out, FwdEntry* e);         \
     bool fir_lookup_c##C(int tap_bucket, int in, FwdEntry* e);                  \
-    bool idft_lookup_c##C(IdftEntry* e);                                         \
+    bool idft_lookup_c##C(FwdEntry* e);                                          \
     int fwd_twiddle_count_c##C();                                                \
     void fwd_twiddles_c##C(float* host_pairs);
 PPF_DECLARE_C(32)
