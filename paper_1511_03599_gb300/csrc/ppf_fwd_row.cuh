@@ -88,6 +88,28 @@ __device__ __forceinline__ void cp_async_wait_upto(int n) {
     }
 }
 
+// A pair of 8- or 16-bit samples as (re, re) and (im, im): the real parts by the
+// conversion unit, the imaginary parts (sign bit flipped) placed in the low
+// mantissa of 2^23 and the bias taken off by one packed add; both are exact.
+// The conversion unit does 16 lanes a clock, and a batch converts its halo rows
+// again ((L + TM - 1) / L times each sample), so sharing the work pays where L
+// is small: C = 4096 int8 T = 16 196 -> 217 GS/s, T = 4 335 -> 358, T = 8 277 -> 281,
+// int16 T = 8 242 -> 256, C = 1024 int8 T = 16 326 -> 335.
+template <int IN, class W>
+__device__ __forceinline__ void cvt_mixed(W w, unsigned long long& re, unsigned long long& im) {
+    if constexpr (IN == IN_CI8) {
+        re = pk2((float)(int8_t)(w & 0xff), (float)(int8_t)((w >> 16) & 0xff));
+        const uint32_t u = w ^ 0x80808080u;
+        im = add2(pk2(__uint_as_float(__byte_perm(u, 0x4B000000u, 0x7441)), __uint_as_float(__byte_perm(u, 0x4B000000u, 0x7443))),
+                  pk2(-8388736.f, -8388736.f));
+    } else {
+        re = pk2((float)(int16_t)(w.x & 0xffff), (float)(int16_t)(w.y & 0xffff));
+        im = add2(pk2(__uint_as_float(__byte_perm(w.x ^ 0x80008000u, 0x4B000000u, 0x7432)),
+                      __uint_as_float(__byte_perm(w.y ^ 0x80008000u, 0x4B000000u, 0x7432))),
+                  pk2(-8421376.f, -8421376.f));
+    }
+}
+
 // R0-point DFT (sign -i) of two neighbouring columns at once: re[a], im[a]
 // hold the real and imaginary parts of both columns.
 template <int R0>
@@ -185,6 +207,9 @@ struct RowShape {
     static constexpr int NR = !RING ? 0 : fits(NR_MAX, true) ? NR_MAX : NR_MIN;
     static constexpr int AHEAD = NR == NR_MAX ? 2 : 1;                   // batches whose rows the ring holds
     static constexpr bool TW_SMEM = RING ? fits(NR, true) : true;
+    // 8/16-bit pairs are converted by two units (cvt_mixed); not with 16 taps held
+    // in registers (C = 2048 T = 16: -1 %)
+    static constexpr bool MIXED = PAIR && IN != IN_CF32 && (L <= 5 || TM <= 8);
     // STAGE: each thread copies the rows of its columns ahead of their use
     // with cp.async into NCH groups of GR slots of its own
     static constexpr int CB = BIN * (PAIR ? 2 : 1);                      // bytes of one copy
@@ -347,7 +372,9 @@ __device__ __forceinline__ bool row_range(const FwdArgs& args, const void* in, v
                     int s = base + seg + i;
                     s = s >= NR ? s - NR : s;
                     const unsigned char* p = ring + s * S::ROWB + off;
-                    if constexpr (PAIR) {
+                    if constexpr (S::MIXED && IN == IN_CI8) cvt_mixed<IN>(*reinterpret_cast<const uint32_t*>(p), x0, x1);
+                    else if constexpr (S::MIXED) cvt_mixed<IN>(*reinterpret_cast<const uint2*>(p), x0, x1);
+                    else if constexpr (PAIR) {
                         const float4 v = load_pair_smem<IN>(p);
                         x0 = pk2(v.x, v.z);
                         x1 = CONJ ? pk2(-v.y, -v.w) : pk2(v.y, v.w);
@@ -358,7 +385,12 @@ __device__ __forceinline__ bool row_range(const FwdArgs& args, const void* in, v
                 } else if constexpr (!S::STAGE) {
                     const long long r = row0 + seg + i;
                     const bool ok = inside || r < n_raw;
-                    if constexpr (PAIR) {
+                    const unsigned char* p = static_cast<const unsigned char*>(in) + (size_t)(r * C + a * M + col) * BIN;
+                    if constexpr (S::MIXED && IN == IN_CI8) {
+                        cvt_mixed<IN>(ok ? __ldg(reinterpret_cast<const uint32_t*>(p)) : 0u, x0, x1);
+                    } else if constexpr (S::MIXED) {
+                        cvt_mixed<IN>(ok ? __ldg(reinterpret_cast<const uint2*>(p)) : make_uint2(0u, 0u), x0, x1);
+                    } else if constexpr (PAIR) {
                         const float4 v = ok ? load_pair_global<IN>(in, r * C + a * M + col) : make_float4(0.f, 0.f, 0.f, 0.f);
                         x0 = pk2(v.x, v.z);
                         x1 = CONJ ? pk2(-v.y, -v.w) : pk2(v.y, v.w);
