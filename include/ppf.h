@@ -194,7 +194,7 @@ ppf_status ppf_update_taps(ppf_plan_t plan, const float* taps_dev, ppf_stream_t 
  *   in [64, 4096]), T[i] <= 16 taps, n_spectra[i] output spectra and taps_host[i]
  *   (C[i]*T[i] FP32, tap-major; read during the call).  Complex int8 input and
  *   complex FP32 output only (else UNSUPPORTED).  The plan cuts every beam
- *   into tiles of about 2^20 samples, sorts them largest first into a wide
+ *   into tiles of about 2^13 to 2^20 samples (about 24 per SM), sorts them largest first into a wide
  *   (C >= 1024) and a narrow queue and keeps taps, twiddles, descriptors,
  *   tiles, two work-queue counters and a status word in device memory it
  *   allocates.  Synchronous.

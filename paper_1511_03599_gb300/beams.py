@@ -135,7 +135,7 @@ def _time(fn, reps=3):
     return a.elapsed_time(b) / reps
 
 
-def autotune(bs: BeamSet, tile_candidates=(1 << 18, 1 << 19, 1 << 20, 1 << 21, 1 << 22),
+def autotune(bs: BeamSet, tile_candidates=(1 << 14, 1 << 16, 1 << 17, 1 << 18, 1 << 19, 1 << 20, 1 << 21, 1 << 22),
              cache_path: str | None = DEFAULT_CACHE, use_cache: bool = True) -> dict:
     """Pick (tile_samples, ctas_per_sm) for this beam set by timing it; cache the choice."""
     sig = bs.signature()
