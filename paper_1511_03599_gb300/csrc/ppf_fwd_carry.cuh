@@ -79,6 +79,12 @@ struct CarryCand {
     static constexpr int REGS_EST = 4 * B + 4 * (TM - 1) + 4 * TM + 4;
     static constexpr int REGS = REGS_EST <= 64 ? 64 : REGS_EST <= 80 ? 80 : REGS_EST <= 96 ? 96
                               : REGS_EST <= 128 ? 128 : REGS_EST <= 168 ? 168 : 255;
+    // FP32 input whose taps fill the bucket: a FIR without the per-tap check that
+    // keeps the bucket's zero taps off the samples.  Where the FIR counts -- 16
+    // taps, and 8 at C = 512 -- (GS/s: C = 256 T = 16 265 -> 354, C = 512 T = 16 250 ->
+    // 324, T = 8 327 -> 384); the shapes at the copy bandwidth lost up to 7 %
+    // (C = 256 T = 8 400 -> 372)
+    static constexpr bool UNCHECKED = IN == IN_CF32 && (TM > 8 || (TM == 8 && C >= 512));
     static constexpr int SMEM_PER_SM = 228 * 1024;
     static constexpr int CTAS_REG = 65536 / (NT * REGS);
     static constexpr int CTAS_SMEM = SMEM_PER_SM / (BASE + TWBYTES + 1024);
@@ -259,6 +265,8 @@ __device__ __forceinline__ bool carry_range(const FwdArgs& args, const void* in,
 #pragma unroll
             for (int j = 0; j < B; ++j) acc[j][0] = acc[j][1] = 0ull;
             float4 nxt[TM > 1 ? TM - 1 : 1];
+            auto fir = [&](auto check_tag) {
+                constexpr bool CHECK = decltype(check_tag)::value != 0;   // fp32: keep inf/NaN out of unrelated outputs
 #pragma unroll
             for (int i = 0; i < B + TM - 1; ++i) {
                 float4 x = (i < TM - 1) ? carry[i < TM - 1 ? i : 0]
@@ -269,13 +277,22 @@ __device__ __forceinline__ bool carry_range(const FwdArgs& args, const void* in,
                 for (int j = 0; j < B; ++j) {
                     const int t = i - j;
                     if (t >= 0 && t < TM) {
-                        if (IN != IN_CF32 || t >= D) {      // fp32: keep inf/NaN out of unrelated outputs
+                        if (!CHECK || t >= D) {
                             ffma2(acc[j][0], h0[t], x01);
                             ffma2(acc[j][1], h1[t], x23);
                         }
                     }
                 }
                 if (i >= B) nxt[i - B] = x;
+            }
+            };
+            if constexpr (IN != IN_CF32) {
+                fir(ic<0>{});
+            } else if constexpr (S::UNCHECKED) {
+                if (D == 0) fir(ic<0>{});
+                else fir(ic<1>{});
+            } else {
+                fir(ic<1>{});
             }
 #pragma unroll
             for (int i = 0; i < TM - 1; ++i) carry[i] = nxt[i];
