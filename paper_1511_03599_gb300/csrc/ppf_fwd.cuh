@@ -343,13 +343,14 @@ struct HalfGroup {
 // INV: the unnormalised inverse DFT (sign +i) computed as conj(DFT(conj(.)));
 // its last stage writes the result back into the spectrum's own row of
 // ybuf in natural order instead of to global memory.
+// reads_done: a barrier each warp arrives on once it has read its last stage's input.
 // CONJ: the last stage stores conjugates (the other half of an inverse DFT
 // whose caller conjugates the input).
 template <int C, int B, int NT, int P, int OUT, bool TW_SMEM, int SPW = 0, bool INV = false, bool SMEM_OUT = false,
           int LAYOUT = 0, class GRP = CtaGroup, bool OOP = false, bool CONJ = false>
 __device__ __forceinline__ void fft_stage(float2* __restrict__ ybuf, const float2* __restrict__ tws,
                                           void* __restrict__ out, long long sb, long long vlo, long long vhi,
-                                          float2* __restrict__ dbuf = nullptr) {
+                                          float2* __restrict__ dbuf = nullptr, uint64_t* reads_done = nullptr) {
     constexpr int NST = fft_stages(C);
     constexpr int R = fft_radix(C, P);
     constexpr int NP = fft_n(C, P);
@@ -402,6 +403,7 @@ __device__ __forceinline__ void fft_stage(float2* __restrict__ ybuf, const float
     // global memory, and the caller orders the buffer's next writer after
     // these reads with a barrier of its own
     if constexpr (!OOP) sync();
+    if (P + 1 == NST && reads_done != nullptr && (gtid & 31) == 0) mbar_arrive_cta(reads_done);
 #pragma unroll
     for (int it = 0; it < IPT; ++it) {
         const int item = wid + it * WORKERS;

@@ -85,6 +85,7 @@ struct CarryCand {
     // 324, T = 8 327 -> 384); the shapes at the copy bandwidth lost up to 7 %
     // (C = 256 T = 8 400 -> 372)
     static constexpr bool UNCHECKED = IN == IN_CF32 && (TM > 8 || (TM == 8 && C >= 512));
+    static constexpr bool FREE_RUN = C == 1024 || (C == 512 && ((IN == IN_CI8 && TM <= 4) || (IN == IN_CI16 && TM > 8)));
     static constexpr int SMEM_PER_SM = 228 * 1024;
     static constexpr int CTAS_REG = 65536 / (NT * REGS);
     static constexpr int CTAS_SMEM = SMEM_PER_SM / (BASE + TWBYTES + 1024);
@@ -160,8 +161,18 @@ __device__ __forceinline__ bool carry_range(const FwdArgs& args, const void* in,
     float2* ybuf = reinterpret_cast<float2*>(smem);
     float2* tw_s = reinterpret_cast<float2*>(smem + S::YBYTES);
     unsigned char* ring = smem + S::RING_OFF;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(ring + 2 * S::SLOTB);     // 3 barriers
-    volatile int* sflag = reinterpret_cast<volatile int*>(bars + 3);
+    // FREE: one CTA-wide barrier per batch (the filtered batch is complete) instead
+    // of two.  Every thread waits for the raw slot itself, and a counted barrier
+    // tells when all warps have read the batch, so a warp done with its spectra
+    // filters the next batch while others still transform.  At C = 1024, where one
+    // CTA of 16 warps fills the SM (int8 T = 8 385 -> 417 GS/s, T = 4 418 -> 458), and
+    // at C = 512 with few int8 taps (T = 4 436 -> 462, T = 1 470 -> 503) or 16 int16 taps
+    // (341 -> 352); elsewhere it measured -8 .. +1 % (the waits cost registers where
+    // those are short, and CTAs that share an SM already fill each other's gaps).
+    constexpr bool FREE = S::FREE_RUN && !FIRONLY;
+    constexpr int NBAR = FREE ? 4 : 3;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(ring + 2 * S::SLOTB);     // slots 0 and 1, never, ybuf read (FREE)
+    volatile int* sflag = reinterpret_cast<volatile int*>(bars + NBAR);
 
     const int tid = GRP::tid();
     const int cp = tid;                              // channel pair
@@ -200,6 +211,7 @@ __device__ __forceinline__ bool carry_range(const FwdArgs& args, const void* in,
     constexpr bool EARLY = IN == IN_CF32;
     if (tid == 0) {
         for (int i = 0; i < 3; ++i) mbar_init(&bars[i], 1);
+        if constexpr (FREE) mbar_init(&bars[NBAR - 1], S::NWARP);
         fence_mbar_init();
         *sflag = 0;
         if constexpr (MULTI) fence_proxy_async_smem();   // the slots were last read by the previous range
@@ -240,8 +252,20 @@ __device__ __forceinline__ bool carry_range(const FwdArgs& args, const void* in,
         if (nraw_b > 1) issue(1);
     }
 
+    bool dead = false;                               // FREE: a wait of this thread gave up
     for (long long k = 0; k < nraw_b; ++k) {
         // ------------------------------------------------ wait for slot k
+        if constexpr (FREE) {
+            if (!dead) {
+                bool ok = rows_of(k) == 0 || mbar_wait_bounded(&bars[k & 1], (uint32_t)((k >> 1) & 1), kWaitLimitNs);
+                if (k == 0 && tid == 0 && (args.flags & FWD_INJECT_TIMEOUT))     // a barrier nothing arrives on
+                    ok = ok && mbar_wait_bounded(&bars[2], 0, kInjectedWaitNs);
+                if (!ok) {
+                    atomicExch(args.err, 1);
+                    dead = true;
+                }
+            }
+        } else {
         if (tid == 0) {
             bool ok = rows_of(k) == 0 || mbar_wait_bounded(&bars[k & 1], (uint32_t)((k >> 1) & 1), kWaitLimitNs);
             if (k == 0 && (args.flags & FWD_INJECT_TIMEOUT))     // a barrier nothing arrives on
@@ -256,6 +280,7 @@ __device__ __forceinline__ bool carry_range(const FwdArgs& args, const void* in,
         }
         GRP::sync();
         if (*sflag) return false;
+        }
         // ---------------------------------------------------------- FIR
         // sequence x_i: i < TM-1 carried rows, then the B rows of slot k.
         // output j = sum_{t < TM} h'[t] x_{j+t}
@@ -308,6 +333,12 @@ __device__ __forceinline__ bool carry_range(const FwdArgs& args, const void* in,
                     }
                 }
             } else {
+                if constexpr (FREE) {
+                    if (k > 0 && !dead && !mbar_wait_bounded(&bars[NBAR - 1], (uint32_t)((k - 1) & 1), kWaitLimitNs)) {
+                        atomicExch(args.err, 1);
+                        dead = true;
+                    }
+                }
 #pragma unroll
                 for (int j = 0; j < B; ++j) {
                     const float2 a = upk2(acc[j][0]), b = upk2(acc[j][1]);
@@ -315,7 +346,16 @@ __device__ __forceinline__ bool carry_range(const FwdArgs& args, const void* in,
                 }
             }
         }
-        GRP::sync();
+        if constexpr (FREE) {
+            if (__syncthreads_or(dead)) {
+                if (tid == 0)
+                    for (long long j = k; j < k + 2 && j < nraw_b; ++j)
+                        if (rows_of(j) > 0) mbar_wait_bounded(&bars[j & 1], (uint32_t)((j >> 1) & 1), kWaitLimitNs);
+                return false;
+            }
+        } else {
+            GRP::sync();
+        }
         // slot k is free: refill it with raw batch k+2
         if (tid == 0 && k + 2 < nraw_b) {
             fence_proxy_async_smem();
@@ -326,14 +366,14 @@ __device__ __forceinline__ bool carry_range(const FwdArgs& args, const void* in,
             const long long sb = (lo + k) * B + sh - (T - 1);     // output spectrum of batch row 0
             static_for<NST>([&](auto p) {
                 fft_stage<C, B, NT, decltype(p)::value, OUT, S::TW_SMEM, S::SPW, false, false, S::LAYOUT, GRP, false, CONJ>(
-                    ybuf, tws, out, sb, vlo, vhi);
+                    ybuf, tws, out, sb, vlo, vhi, nullptr, FREE ? &bars[NBAR - 1] : nullptr);
             });
         }
     }
     if constexpr (MULTI) {
         GRP::sync();                                 // every thread is past its last wait
         if (tid == 0)
-            for (int i = 0; i < 3; ++i) mbar_inval(&bars[i]);
+            for (int i = 0; i < NBAR; ++i) mbar_inval(&bars[i]);
     }
     return true;
 }
