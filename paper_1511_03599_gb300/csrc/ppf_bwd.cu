@@ -53,8 +53,8 @@ bool bwd_lookup(int C, int tm, int in, BwdEntry* e) {
 cudaError_t bwd_reduce(const float* partials, int nparts, int T, int TM, int C, const int* err, float* grad_h,
                        cudaStream_t st) {
     const int TC = T * C;
-    pfb_bwd_reduce_kernel<<<(TC + 31) / 32, dim3(32, kReduceLanes), 0, st>>>(partials, nparts, TC, TM * C, err, grad_h);
-    return cudaPeekAtLastError();
+    return launch_early(pfb_bwd_reduce_kernel, (TC + 31) / 32, dim3(32, kReduceLanes), 0, st, partials, nparts, TC, TM * C,
+                        err, grad_h);
 }
 
 template <int IN, int NCT, bool GX, bool GH>
@@ -64,8 +64,7 @@ static cudaError_t grad_launch(const AdjArgs& a, const AdjMaps& m, int parts, cu
     const cudaError_t ce = cudaFuncSetAttribute(pfb_bwd_grad_kernel<IN, NCT, GX, GH>,
                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, S::smem(PPF_MAX_TAPS));
     if (ce != cudaSuccess) return ce;
-    pfb_bwd_grad_kernel<IN, NCT, GX, GH><<<dim3(parts, a.C / NCT), S::NT, smem, st>>>(a, m.g, m.x, m.taps);
-    return cudaPeekAtLastError();
+    return launch_early(pfb_bwd_grad_kernel<IN, NCT, GX, GH>, dim3(parts, a.C / NCT), S::NT, smem, st, a, m.g, m.x, m.taps);
 }
 
 template <int IN, int NCT>

@@ -306,6 +306,7 @@ static __global__ void __launch_bounds__(32 * kReduceLanes)
 pfb_bwd_reduce_kernel(const float* __restrict__ partials, int nparts, int TC, int TMC, const int* __restrict__ err,
                       float* __restrict__ grad_h) {
     __shared__ float sums[kReduceLanes][32];
+    grid_dependency_wait();                             // launched by launch_early
     const int i = blockIdx.x * 32 + threadIdx.x;
     float s = 0.f;
     if (i < TC) {

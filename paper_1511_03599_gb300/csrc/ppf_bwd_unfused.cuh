@@ -130,6 +130,7 @@ pfb_bwd_grad_kernel(AdjArgs a, const __grid_constant__ CUtensorMap g_map, const 
     volatile int* sdead = reinterpret_cast<volatile int*>(full + 2 * NS);
     float* ghs = reinterpret_cast<float*>(smem + S::GH_OFF);              // [T][NCT]
 
+    grid_dependency_wait();                                               // launched by launch_early
     const int tid = threadIdx.x, lane = tid & 31;
     const int c0 = blockIdx.y * NCT;
     const int T = a.T;

@@ -355,6 +355,10 @@ __device__ __forceinline__ void tma_load_1d_once(void* dst_smem, const void* src
         "l"(src_gmem), "r"(bytes), "r"(smem_addr(bar)), "l"(pol)
         : "memory");
 }
+// Wait until the kernels before this one in the stream have ended and their
+// writes are visible (returns at once unless launched by launch_early).
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // One box of a tensor map global -> shared (tile mode) completing on `bar`;
 // the smem address is 128-byte aligned, x * element size a multiple of 16.
 __device__ __forceinline__ void tma_load_box2(void* dst_smem, const void* map, int x, int y, uint64_t* bar) {

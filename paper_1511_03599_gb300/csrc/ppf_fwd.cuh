@@ -960,16 +960,14 @@ inline cudaError_t fwd_launch(const FwdArgs& a, int grid, cudaStream_t st) {
 template <int C, int TM, int IN, int OUT>
 inline cudaError_t row_small_launch(const FwdArgs& a, int grid, cudaStream_t st) {
     using S = RowShape<C, TM, IN, 4>;
-    pfb_fwd_row_kernel<C, TM, IN, OUT, 4><<<grid, S::NT, S::SMEM, st>>>(a);
-    return cudaPeekAtLastError();
+    return launch_early(pfb_fwd_row_kernel<C, TM, IN, OUT, 4>, grid, S::NT, S::SMEM, st, a);
 }
 
 // The carry kernel's form for short ranges (FwdEntry::short_*).
 template <int C, int TM, int IN, int OUT>
 inline cudaError_t carry_short_launch(const FwdArgs& a, int grid, cudaStream_t st) {
     using S = CarryShape<C, TM, IN>;
-    pfb_fwd_carry_kernel<C, TM, IN, OUT, false, true><<<grid, S::NT, S::SMEM, st>>>(a);
-    return cudaPeekAtLastError();
+    return launch_early(pfb_fwd_carry_kernel<C, TM, IN, OUT, false, true>, grid, S::NT, S::SMEM, st, a);
 }
 
 // FIR-only ablation kernels (carry shapes only), output complex FP32 rows.

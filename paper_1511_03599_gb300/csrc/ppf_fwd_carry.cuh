@@ -387,6 +387,7 @@ pfb_fwd_carry_kernel(FwdArgs args) {
     using S = CarryShape<C, TM, IN>;
     constexpr int B = S::B, BIN = S::BIN;
     extern __shared__ __align__(128) unsigned char smem[];
+    if constexpr (SHORT) grid_dependency_wait();     // launched by launch_early
     const long long nbt = (args.n_spectra + B - 1) / B;
     const int cps = (int)(gridDim.x / args.n_streams);   // CTAs per stream (the grid is a multiple)
     const int strm = blockIdx.x / cps, bx = blockIdx.x - strm * cps;

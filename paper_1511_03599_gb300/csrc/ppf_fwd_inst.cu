@@ -110,6 +110,11 @@ static cudaError_t launch_kernel(const FwdArgs& a, int grid, cudaStream_t st) {
     return cudaPeekAtLastError();
 }
 
+template <auto KERNEL, int NT, int SMEM>
+static cudaError_t launch_kernel_early(const FwdArgs& a, int grid, cudaStream_t st) {
+    return launch_early(KERNEL, grid, NT, SMEM, st, a);
+}
+
 // The inverse DFT of the three-pass adjoint: the forward kernels with T = 1 and
 // conjugation; the small batches wherever the forward has them.
 template <int C>
@@ -136,7 +141,7 @@ static bool make_idft(FwdEntry* e) {
             e->fn = reinterpret_cast<const void*>(k);
             e->launch = &launch_kernel<k, S::NT, S::SMEM>;
             e->short_fn = reinterpret_cast<const void*>(ks);
-            e->short_launch = &launch_kernel<ks, S::NT, S::SMEM>;
+            e->short_launch = &launch_kernel_early<ks, S::NT, S::SMEM>;
         } else {
             using S = RowShape<C, 1, IN_CF32>;
             constexpr auto k = &pfb_fwd_row_kernel<C, 1, IN_CF32, OUT_CF32, 1, true>;
@@ -152,7 +157,7 @@ static bool make_idft(FwdEntry* e) {
         e->small_batch = M::B;
         e->small_smem = M::SMEM;
         e->small_fn = reinterpret_cast<const void*>(km);
-        e->small_launch = &launch_kernel<km, M::NT, M::SMEM>;
+        e->small_launch = &launch_kernel_early<km, M::NT, M::SMEM>;
         return true;
     }
 }

@@ -36,6 +36,7 @@
 #pragma once
 
 #include "ppf_fwd_carry.cuh"
+#include "ppf_launch.h"
 #include "ppf_tmap.h"
 
 namespace ppf {
@@ -85,6 +86,7 @@ pfb_fwd_longtap_kernel(FwdArgs args, const __grid_constant__ CUtensorMap in_map,
     uint64_t* inj = full + 2 * NS;                                       // never completed (testing aid)
     volatile int* sdead = reinterpret_cast<volatile int*>(full + 2 * NS + 1);
 
+    if constexpr (DIV > 1) grid_dependency_wait();   // launched by launch_early
     const int tid = threadIdx.x, lane = tid & 31;
     const long long n_spectra = args.n_spectra;
     const int T = args.T;                        // 17 .. 64
@@ -267,8 +269,12 @@ inline cudaError_t longtap_launch(const FwdArgs& a, int grid, cudaStream_t st) {
     CUtensorMap in_map, tap_map;
     const cudaError_t ce = longtap_maps(a, C, S::BIN, S::NCT, &in_map, &tap_map);
     if (ce != cudaSuccess) return ce;
-    pfb_fwd_longtap_kernel<C, IN, OUT, DIV><<<grid, S::NT, S::SMEM, st>>>(a, in_map, tap_map);
-    return cudaPeekAtLastError();
+    if constexpr (DIV > 1) {
+        return launch_early(pfb_fwd_longtap_kernel<C, IN, OUT, DIV>, grid, S::NT, S::SMEM, st, a, in_map, tap_map);
+    } else {
+        pfb_fwd_longtap_kernel<C, IN, OUT, DIV><<<grid, S::NT, S::SMEM, st>>>(a, in_map, tap_map);
+        return cudaPeekAtLastError();
+    }
 }
 
 }  // namespace ppf

@@ -650,6 +650,7 @@ template <int C, int TM, int IN, int OUT, int DIV = 1, bool CONJ = false>
 __global__ void __launch_bounds__(kRowThreads, 1) pfb_fwd_row_kernel(FwdArgs args) {
     using S = RowShape<C, TM, IN, DIV>;
     extern __shared__ __align__(128) unsigned char smem[];
+    if constexpr (DIV > 1) grid_dependency_wait();   // launched by launch_early
     BatchShare share((args.n_spectra + S::B - 1) / S::B, args.n_streams, blockIdx.x, gridDim.x);
     long long strm, lo, hi;
     while (share.next(strm, lo, hi)) {
