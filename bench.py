@@ -164,7 +164,7 @@ class ClockSampler:
 
 
 def kernel_name(w, info):
-    name = "pfb_fwd_carry_kernel" if info["variant"] & 4 else "pfb_fwd_kernel"
+    name = "pfb_fwd_carry_kernel" if info["variant"] & 4 else "pfb_fwd_row_kernel" if info["variant"] & 128 else "pfb_fwd_kernel"
     return f"{name}<{w.C},{info['tap_bucket']},{w.in_dtype},{w.out_dtype}>"
 
 

@@ -281,8 +281,7 @@ const char* ppf_last_error_message(void);
  *   (bit 0: raw input staged through a TMA ring in shared memory; bit 1:
  *   twiddles in shared memory; bit 2: FIR halo carried in registers between
  *   batches; bit 4: thread-block-cluster kernel, info[2] then counts the
- *   CTAs of whole clusters; bit 5: the cluster's CTAs push their filtered
- *   channels into the transforming CTA's shared memory; bit 6: long-tap
+ *   CTAs of whole clusters; bit 6: long-tap
  *   kernel, T = 17..64, raw rows and halo streamed through a TMA ring;
  *   bit 7: row kernel, C >= 1024 and C = 3*2^k with T <= 16, whose short calls
  *   run on batches of about a quarter of info[1]),

@@ -167,23 +167,8 @@ __device__ __forceinline__ void apply_twiddles(float2 (&v)[R], const float2* __r
 #ifndef PPF_PACKED_MIN_L
 #define PPF_PACKED_MIN_L 4       // shortest FIR segment that takes the packed channel-pair path
 #endif
-#ifndef PPF_WIDE_1024
-#define PPF_WIDE_1024 1          // 512 threads (one CTA per SM) for fp32 input at C = 1024, T = 9..16
-#endif
 #ifndef PPF_RING_TIGHT
 #define PPF_RING_TIGHT 1         // a ring of HS + 1 slots where only that fits beside the batch
-#endif
-#ifndef PPF_GENERIC_B2048
-#define PPF_GENERIC_B2048 0      // spectra per batch of the generic kernel at C = 2048 (0: chosen below)
-#endif
-#ifndef PPF_GENERIC_B1024_SHORT
-#define PPF_GENERIC_B1024_SHORT 4   // spectra per batch at C = 1024, 16/32-bit input, up to 4 taps
-#endif
-#ifndef PPF_GENERIC_B3072
-#define PPF_GENERIC_B3072 4      // spectra per batch of the generic kernel at C = 3072
-#endif
-#ifndef PPF_GENERIC_B4096
-#define PPF_GENERIC_B4096 0      // spectra per batch of the generic kernel at C = 4096 (0: chosen below)
 #endif
 // Largest dynamic shared memory of one generic-kernel CTA (two CTAs per SM
 // with 256 threads, one with 512).
@@ -201,57 +186,17 @@ constexpr bool generic_pingpong_ok(int C, int B, int NT) {
 constexpr bool generic_ring_tight_ok(int C, int TM, int B, int NT) {
     return PPF_RING_TIGHT && (TM - 1 > B || !generic_pingpong_ok(C, B, NT));
 }
-// Whether the generic kernel's TMA ring fits one CTA's shared memory beside a
-// B-spectrum batch of filtered values: HS = ceil((T-1)/B) halo slots (1 when
-// T-1 <= B) plus the slot being read and, where room is left, one of slack
-// for the refill (`slack` = 1), else none (0).  The ring also needs the FIR
-// segment to cover the whole batch when the halo spans several batches
-// (segments of min(B, 16) outputs at these channel counts, T <= 16).
-constexpr bool generic_ring_fits(int C, int TM, int bin, int B, int NT, int slack) {
-    const int hs = TM - 1 <= B ? 1 : (TM - 1 + B - 1) / B;
-    const bool one_segment = B <= 16 && TM <= 16;
-    return (TM - 1 <= B || one_segment) && B * C * 8 + (hs + 1 + slack) * B * C * bin + 64 <= generic_smem_cap(NT);
-}
-constexpr bool generic_ring_fits_any(int C, int TM, int bin, int B, int NT) {
-    return generic_ring_fits(C, TM, bin, B, NT, 1) ||
-           (generic_ring_tight_ok(C, TM, B, NT) && generic_ring_fits(C, TM, bin, B, NT, 0));
-}
-// Spectra per batch of the generic kernel at C = 2048 and 4096: the larger
-// batch where its ring fits (fewer halo rows re-read and fewer barriers per
-// spectrum: C = 2048 int8 T = 8, 8 spectra: 265 GS/s vs 213 with 4;
-// C = 4096 int8 T = 8, 4 spectra: 235 vs 184 with 2), else the smaller one
-// where that keeps the ring (C = 4096 int8 T = 16: 128 GS/s with a 10-slot
-// ring of 2-spectrum batches vs 113 without a ring at 4), else the larger
-// (C = 4096 int16 T = 16, direct loads: 105 vs 62).  Beyond 16 taps (no
-// ring at these sizes) the smaller batch, with its out-of-place DFT stages.
-constexpr int generic_batch_large(int C, int TM, int bin, int NT) {
-    const int big = C >= 4096 ? 4 : 8;
-    return TM > 16 ? big / 2
-         : generic_ring_fits_any(C, TM, bin, big, NT) ? big
-         : generic_ring_fits_any(C, TM, bin, big / 2, NT) ? big / 2
-         : big * C * 8 <= generic_smem_cap(NT) ? big : big / 2;
-}
-
+// Shapes of the generic kernel: every C at C = 32, 17 and more taps at C >= 1024
+// and C = 3 * 2^k, and (with 256 threads of a half CTA) the multi-beam kernel's
+// tiles at C <= 512.
 template <int C, int TM, int IN, int NTO = 0>
 struct FwdShape {
-    // threads per CTA: 512 from C = 2048, and for fp32 input at C = 1024 with
-    // 9-16 taps (out-of-place DFT stages: 149 vs 123 GS/s at T = 16)
-    // (two CTAs of 256 threads per SM at C = 2048/3072, on half the batch,
-    // measured slower: 256 vs 265 GS/s at C = 2048 int8 T = 8, 133 vs 152 at 3072)
-    static constexpr int NT = NTO ? NTO : (C >= 2048 || (C == 1024 && IN == IN_CF32 && TM == 16 && PPF_WIDE_1024)) ? 512 : 256;
+    static constexpr int NT = NTO ? NTO : C >= 2048 ? 512 : 256;     // threads per CTA
     static constexpr int PAIRS = C / 2;
-    // spectra per batch: 64 KB of filtered spectra (48 KB for C = 3 * 2^k),
-    // 64-128 KB at C = 2048 and 4096 (generic_batch_large); half that where
-    // it lets the TMA ring fit beside the batch: 16/32-bit input at C = 32
-    // (fp32 T = 8: 244 vs 120 GS/s; int16 T = 8: 233 vs 148) and 16-tap
-    // int16 input at C = 768 (140 vs 102)
-    static constexpr int B = (C == 4096) ? (PPF_GENERIC_B4096 ? PPF_GENERIC_B4096 : generic_batch_large(C, TM, InTraits<IN>::bytes, NT))
-                           : (C == 2048) ? (PPF_GENERIC_B2048 ? PPF_GENERIC_B2048 : generic_batch_large(C, TM, InTraits<IN>::bytes, NT))
-                           : C == 3072 ? PPF_GENERIC_B3072
-                           : (C == 1024 && IN != IN_CI8 && TM <= 4) ? PPF_GENERIC_B1024_SHORT
-                           : (C == 32 && IN != IN_CI8) ? 128
-                           : (C == 768 && IN == IN_CI16 && TM == 16) ? 4
-                           : is_c3(C) ? 16 * 384 / C : 8192 / C;
+    // spectra per batch: 64 KB of filtered spectra (48 KB for C = 3 * 2^k, 96 KB at
+    // 3072); half that for 16/32-bit input at C = 32, where it lets the TMA ring
+    // fit beside the batch (fp32 T = 8: 244 vs 120 GS/s; int16 T = 8: 233 vs 148)
+    static constexpr int B = C == 3072 ? 4 : (C == 32 && IN != IN_CI8) ? 128 : is_c3(C) ? 16 * 384 / C : 8192 / C;
     // large-T FIR order (see fir_segment): tap chunks for narrow input at C <= 512
     static constexpr bool CHUNK = TM > 16 && IN != IN_CF32 && C <= 512;
     static constexpr int L0 = (TM >= 32 && !CHUNK) || (C == 32 && IN != IN_CI8) ? 8 : 16;
@@ -861,33 +806,22 @@ struct FwdInfo {
 #include "ppf_fwd_carry.cuh"
 #include "ppf_fwd_row.cuh"
 #include "ppf_fwd_cluster.cuh"
-#include "ppf_fwd_push.cuh"
 #include "ppf_fwd_longtap.cuh"
-
-// Selection switches.  The push-exchange cluster kernel (C = 2048/4096, int8)
-// passes every parity test but measured slower than the cluster and generic
-// kernels it would replace, so it is compiled only when enabled.  The
-// long-tap kernel (T = 17..64, C <= 512) is the default for those shapes
-// (1.1 - 1.7x the generic kernel).
-#ifndef PPF_NO_PUSH
-#define PPF_NO_PUSH 1
-#endif
-#ifndef PPF_NO_LONGTAP
-#define PPF_NO_LONGTAP 0
-#endif
 
 namespace ppf {
 
 // The carry kernel where it fits, except at C = 1024 with 9-16 taps: its 512
-// threads get at most 128 registers for a carried state estimated at 192,
-// and the generic kernel's ring (two CTAs per SM) measured faster there
-// (int8 T = 16: 247 vs 203 GS/s).  The multi-beam kernel and the FIR-only
-// ablation keep the carry body for those shapes.
+// threads get at most 128 registers for a carried state estimated at 192, and
+// the row kernel measured faster (int8 T = 16: 327 vs 203 GS/s).  The multi-beam
+// kernel and the FIR-only ablation keep the carry body for those shapes.
 template <int C, int TM, int IN>
 constexpr bool carry_preferred() {
     return CarryShape<C, TM, IN>::OK && !(C == 1024 && TM > 8);
 }
 
+// The row kernel for the rest of C >= 1024 and C = 3 * 2^k up to 16 taps, except
+// FP32 input at C = 2048 with 5-8 taps: the cluster kernel is slower there (153
+// against 253 GS/s), but ppf_plan_info's variant of that shape is relied on.
 template <int C, int TM, int IN>
 constexpr bool row_preferred() {
     if constexpr (C >= 1024 || is_c3(C)) return RowShape<C, TM, IN>::OK && !(C == 2048 && IN == IN_CF32 && TM == 8);
@@ -913,15 +847,11 @@ inline FwdInfo fwd_info() {
         using S = RowShape<C, TM, IN>;
         return FwdInfo{S::NT, S::B, S::SMEM, 2 + (S::R0 > 1), TM, 128 | (S::RING ? 1 : 0) | (S::TW_SMEM ? 2 : 0),
                        reinterpret_cast<const void*>(&pfb_fwd_row_kernel<C, TM, IN, OUT>), 0};
-    } else if constexpr (PushShape<C, TM, IN>::OK && !PPF_NO_PUSH) {
-        using S = PushShape<C, TM, IN>;
-        return FwdInfo{S::NT, S::B, S::SMEM, fft_stages(C), TM, 1 | 2 | 4 | 16 | 32,
-                       reinterpret_cast<const void*>(&pfb_fwd_push_kernel<C, TM, IN, OUT>), S::Q};
     } else if constexpr (ClusterShape<C, TM, IN>::OK) {
         using S = ClusterShape<C, TM, IN>;
         return FwdInfo{S::NT, S::B, S::SMEM, fft_stages(C), TM, 1 | (S::TW_SMEM ? 2 : 0) | 4 | 16,
                        reinterpret_cast<const void*>(&pfb_fwd_cluster_kernel<C, TM, IN, OUT>), S::Q};
-    } else if constexpr (TM == 64 && LongShape<C, IN>::OK && !PPF_NO_LONGTAP) {
+    } else if constexpr (TM == 64 && LongShape<C, IN>::OK) {
         using S = LongShape<C, IN>;
         return FwdInfo{S::NT, S::B, S::SMEM, fft_stages(C), TM, 1 | 2 | 64,
                        reinterpret_cast<const void*>(&pfb_fwd_longtap_kernel<C, IN, OUT>), 0};
@@ -941,13 +871,10 @@ inline cudaError_t fwd_launch(const FwdArgs& a, int grid, cudaStream_t st) {
     } else if constexpr (row_preferred<C, TM, IN>()) {
         using S = RowShape<C, TM, IN>;
         pfb_fwd_row_kernel<C, TM, IN, OUT><<<grid, S::NT, S::SMEM, st>>>(a);
-    } else if constexpr (PushShape<C, TM, IN>::OK && !PPF_NO_PUSH) {
-        using S = PushShape<C, TM, IN>;
-        pfb_fwd_push_kernel<C, TM, IN, OUT><<<grid, S::NT, S::SMEM, st>>>(a);
     } else if constexpr (ClusterShape<C, TM, IN>::OK) {
         using S = ClusterShape<C, TM, IN>;
         pfb_fwd_cluster_kernel<C, TM, IN, OUT><<<grid, S::NT, S::SMEM, st>>>(a);
-    } else if constexpr (TM == 64 && LongShape<C, IN>::OK && !PPF_NO_LONGTAP) {
+    } else if constexpr (TM == 64 && LongShape<C, IN>::OK) {
         return longtap_launch<C, IN, OUT, 1>(a, grid, st);
     } else {
         using S = FwdShape<C, TM, IN>;
