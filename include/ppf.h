@@ -238,7 +238,7 @@ ppf_status ppf_beams_destroy(ppf_beams_t beams);
  *            Exists where the carry kernel's FIR fits (halo in registers):
  *            C in {64, 128, 256, 512} (and 1024 for int8 input), T <= 16
  *            (else UNSUPPORTED); at C = 1024 with 9-16 taps the fused path
- *            itself runs the generic kernel.
+ *            itself runs the row kernel.
  *   ppf_fft: the DFT alone (Eq. 2) of n_spectra rows of C complex FP32 values
  *            at y_dev into out_dev (the plan's output type); runs the fused
  *            kernel with T = 1 and unit taps (exact); its internal plan is
@@ -283,7 +283,7 @@ const char* ppf_last_error_message(void);
  *   batches; bit 4: thread-block-cluster kernel, info[2] then counts the
  *   CTAs of whole clusters; bit 6: long-tap
  *   kernel, T = 17..64, raw rows and halo streamed through a TMA ring;
- *   bit 7: row kernel, C >= 1024 and C = 3*2^k with T <= 16, whose short calls
+ *   bit 7: row kernel, C >= 1024 and C = 3*2^k, whose short calls
  *   run on batches of about a quarter of info[1]),
  *   info[7]=CTAs resident per SM. */
 ppf_status ppf_plan_info(ppf_plan_t plan, int info[8]);

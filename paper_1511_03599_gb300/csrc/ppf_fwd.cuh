@@ -158,45 +158,22 @@ __device__ __forceinline__ void apply_twiddles(float2 (&v)[R], const float2* __r
 #ifndef PPF_TMA_EVICT_FIRST
 #define PPF_TMA_EVICT_FIRST 1
 #endif
-#ifndef PPF_PINGPONG
-#define PPF_PINGPONG 1
-#endif
-#ifndef PPF_PINGPONG_256
-#define PPF_PINGPONG_256 1       // also for 256 threads at C = 1536 (fp32 +43 %; C = 768 lost 1.5 %)
-#endif
 #ifndef PPF_PACKED_MIN_L
 #define PPF_PACKED_MIN_L 4       // shortest FIR segment that takes the packed channel-pair path
-#endif
-#ifndef PPF_RING_TIGHT
-#define PPF_RING_TIGHT 1         // a ring of HS + 1 slots where only that fits beside the batch
 #endif
 // Largest dynamic shared memory of one generic-kernel CTA (two CTAs per SM
 // with 256 threads, one with 512).
 constexpr int generic_smem_cap(int NT) { return (NT == 256 ? 113 * 1024 : 226 * 1024) - 128; }
-// Whether the direct-load mode can run its DFT stages out of place between
-// two spectra buffers (512 threads, or 256 from C = 1536).
-constexpr bool generic_pingpong_ok(int C, int B, int NT) {
-    return PPF_PINGPONG && (NT == 512 || (PPF_PINGPONG_256 && C >= 1536)) && 2 * B * C * 8 <= generic_smem_cap(NT);
-}
-// Whether a ring without the refill slot is allowed: where the halo spans two
-// or more batches, or where the alternative is plain direct loads (no
-// out-of-place mode).  A 2-slot ring lost to the out-of-place mode (C = 3072
-// int16 T = 4: 160 vs 170 GS/s) but beat plain direct loads (C = 1024 fp32
-// T = 4: 218 vs 175).
-constexpr bool generic_ring_tight_ok(int C, int TM, int B, int NT) {
-    return PPF_RING_TIGHT && (TM - 1 > B || !generic_pingpong_ok(C, B, NT));
-}
-// Shapes of the generic kernel: every C at C = 32, 17 and more taps at C >= 1024
-// and C = 3 * 2^k, and (with 256 threads of a half CTA) the multi-beam kernel's
-// tiles at C <= 512.
+// Shapes of the generic kernel: C = 32, and (with 256 threads of a half CTA) the
+// multi-beam kernel's tiles at C <= 512.
 template <int C, int TM, int IN, int NTO = 0>
 struct FwdShape {
-    static constexpr int NT = NTO ? NTO : C >= 2048 ? 512 : 256;     // threads per CTA
+    static constexpr int NT = NTO ? NTO : 256;                       // threads per CTA
     static constexpr int PAIRS = C / 2;
-    // spectra per batch: 64 KB of filtered spectra (48 KB for C = 3 * 2^k, 96 KB at
-    // 3072); half that for 16/32-bit input at C = 32, where it lets the TMA ring
-    // fit beside the batch (fp32 T = 8: 244 vs 120 GS/s; int16 T = 8: 233 vs 148)
-    static constexpr int B = C == 3072 ? 4 : (C == 32 && IN != IN_CI8) ? 128 : is_c3(C) ? 16 * 384 / C : 8192 / C;
+    // spectra per batch: 64 KB of filtered spectra; half that for 16/32-bit input at
+    // C = 32, where it lets the TMA ring fit beside the batch (fp32 T = 8: 244 vs
+    // 120 GS/s; int16 T = 8: 233 vs 148)
+    static constexpr int B = (C == 32 && IN != IN_CI8) ? 128 : 8192 / C;
     // large-T FIR order (see fir_segment): tap chunks for narrow input at C <= 512
     static constexpr bool CHUNK = TM > 16 && IN != IN_CF32 && C <= 512;
     static constexpr int L0 = (TM >= 32 && !CHUNK) || (C == 32 && IN != IN_CI8) ? 8 : 16;
@@ -223,19 +200,11 @@ struct FwdShape {
     static constexpr bool NS_TIGHT_FITS = YBYTES + (HS + 1) * SLOTB + 64 <= CTA_SMEM_MAX;
     static constexpr bool NS_TIGHT_FOR_TW = YBYTES + (HS + 2) * SLOTB + 64 + TWBYTES > CTA_SMEM_MAX &&
                                             YBYTES + (HS + 1) * SLOTB + 64 + TWBYTES <= CTA_SMEM_MAX;
-    static constexpr int NS = (generic_ring_tight_ok(C, TM, B, NT) && NS_TIGHT_FITS &&
+    static constexpr int NS = (NS_TIGHT_FITS &&
                                (YBYTES + (HS + 2) * SLOTB + 64 > CTA_SMEM_MAX || NS_TIGHT_FOR_TW)) ? HS + 1 : HS + 2;
     static constexpr bool RING = (TM - 1 <= B || (G == 1 && TM <= 16)) && (YBYTES + NS * SLOTB + 64 <= CTA_SMEM_MAX);
-    // direct-load mode with 512 threads (and at C = 1536 with 256): two
-    // filtered-spectra buffers, so the DFT stages run out of place (read one
-    // buffer, write the other), one CTA barrier per stage instead of two
-    // (fp32 at C = 3072: 93 -> 131 GS/s, at C = 1536: 94 -> 135); with the
-    // ring the second buffer would push the twiddles out of shared memory,
-    // which measured 1 % slower at C = 4096
-    static constexpr bool PINGPONG = generic_pingpong_ok(C, B, NT) && !RING;
-    static constexpr int YB = PINGPONG ? 2 * YBYTES : YBYTES;        // bytes of the spectra buffers
-    static constexpr bool TW_SMEM = YB + (RING ? NS * SLOTB + 64 : 0) + TWBYTES <= CTA_SMEM_MAX;
-    static constexpr int RING_OFF = YB + (TW_SMEM ? TWBYTES : 0);
+    static constexpr bool TW_SMEM = YBYTES + (RING ? NS * SLOTB + 64 : 0) + TWBYTES <= CTA_SMEM_MAX;
+    static constexpr int RING_OFF = YBYTES + (TW_SMEM ? TWBYTES : 0);
     static constexpr int SMEM = RING_OFF + (RING ? NS * SLOTB + 64 : 0);
     // each thread keeps one channel pair for the whole run: taps stay in registers
     static constexpr bool TAPS_IN_REGS = (FPT == 1) && (TM <= 16) && (NT % PAIRS == 0);
@@ -292,10 +261,10 @@ struct HalfGroup {
 // CONJ: the last stage stores conjugates (the other half of an inverse DFT
 // whose caller conjugates the input).
 template <int C, int B, int NT, int P, int OUT, bool TW_SMEM, int SPW = 0, bool INV = false, bool SMEM_OUT = false,
-          int LAYOUT = 0, class GRP = CtaGroup, bool OOP = false, bool CONJ = false>
+          int LAYOUT = 0, class GRP = CtaGroup, bool CONJ = false>
 __device__ __forceinline__ void fft_stage(float2* __restrict__ ybuf, const float2* __restrict__ tws,
                                           void* __restrict__ out, long long sb, long long vlo, long long vhi,
-                                          float2* __restrict__ dbuf = nullptr, uint64_t* reads_done = nullptr) {
+                                          uint64_t* reads_done = nullptr) {
     constexpr int NST = fft_stages(C);
     constexpr int R = fft_radix(C, P);
     constexpr int NP = fft_n(C, P);
@@ -308,7 +277,6 @@ __device__ __forceinline__ void fft_stage(float2* __restrict__ ybuf, const float
     constexpr bool EXACT = IPT * WORKERS == TOTAL;
     constexpr int SPAN = spec_span<C, LAYOUT>();   // elements per spectrum in ybuf
     static_assert(!(LAYOUT >= 1 && (INV || SMEM_OUT)), "padded or pair-swizzled rows only for the forward stores to HBM");
-    static_assert(!(OOP && (INV || SMEM_OUT || SPW > 0)), "out-of-place stages only for the CTA-wide forward");
     static_assert(EXACT || (SPW == 0 && is_c3(C)) || TOTAL < WORKERS,
                   "items must divide evenly (a warp or CTA may leave threads idle)");
     const int gtid = GRP::tid();
@@ -343,11 +311,8 @@ __device__ __forceinline__ void fft_stage(float2* __restrict__ ybuf, const float
             }
         }
     }
-    // every read of this stage is done before anything is overwritten; OOP
-    // (out of place): a non-last stage writes to dbuf, a last stage stores to
-    // global memory, and the caller orders the buffer's next writer after
-    // these reads with a barrier of its own
-    if constexpr (!OOP) sync();
+    // every read of this stage is done before anything is overwritten
+    sync();
     if (P + 1 == NST && reads_done != nullptr && (gtid & 31) == 0) mbar_arrive_cta(reads_done);
 #pragma unroll
     for (int it = 0; it < IPT; ++it) {
@@ -358,7 +323,7 @@ __device__ __forceinline__ void fft_stage(float2* __restrict__ ybuf, const float
         dft_reg<R>(v[it]);
         if constexpr (P + 1 < NST) {
             apply_twiddles<R, NN, TW_SMEM>(v[it], tws + tw_offset(C, P), b);
-            float2* dst = (OOP ? dbuf : ybuf) + sp * SPAN;
+            float2* dst = ybuf + sp * SPAN;
 #pragma unroll
             for (int k = 0; k < R; ++k) dst[phys<C, P + 1, LAYOUT>((prefix + PP * k) * NN + b)] = v[it][k];
         } else if constexpr (INV) {
@@ -606,8 +571,7 @@ __device__ __forceinline__ bool fwd_range(const FwdArgs& args, const void* in, v
     constexpr int NST = fft_stages(C);
     constexpr bool RING = S::RING;
     float2* ybuf = reinterpret_cast<float2*>(smem);
-    float2* ybuf2 = reinterpret_cast<float2*>(smem + S::YBYTES);        // PINGPONG only
-    float2* tw_s = reinterpret_cast<float2*>(smem + S::YB);
+    float2* tw_s = reinterpret_cast<float2*>(smem + S::YBYTES);
     unsigned char* ring = smem + S::RING_OFF;
     uint64_t* bars = reinterpret_cast<uint64_t*>(ring + NS * S::SLOTB);   // NS + 1 barriers
     volatile int* sflag = reinterpret_cast<volatile int*>(bars + NS + 1);
@@ -734,22 +698,9 @@ __device__ __forceinline__ bool fwd_range(const FwdArgs& args, const void* in, v
             }
         }
         // ---------------------------------------------------------- FFT
-        if constexpr (S::PINGPONG) {
-            // stage p reads buffer p & 1 and writes buffer (p + 1) & 1; the last
-            // stage's reads are ordered before the next batch's FIR writes by the
-            // barrier after the ring wait, or by the one below without a ring
-            static_for<NST>([&](auto p) {
-                constexpr int P = decltype(p)::value;
-                fft_stage<C, B, NT, P, OUT, S::TW_SMEM, 0, false, false, 0, GRP, true>(
-                    (P & 1) ? ybuf2 : ybuf, tws, out, sb, 0, n_spectra, (P & 1) ? ybuf : ybuf2);
-            });
-            if constexpr (!RING) GRP::sync();
-        } else {
-            static_for<NST>([&](auto p) {
-                fft_stage<C, B, NT, decltype(p)::value, OUT, S::TW_SMEM, 0, false, false, 0, GRP>(ybuf, tws, out, sb, 0,
-                                                                                                  n_spectra);
-            });
-        }
+        static_for<NST>([&](auto p) {
+            fft_stage<C, B, NT, decltype(p)::value, OUT, S::TW_SMEM, 0, false, false, 0, GRP>(ybuf, tws, out, sb, 0, n_spectra);
+        });
     }
     if constexpr (RING) {
         // every copy of the range has landed (thread 0 waited for each):

@@ -365,8 +365,8 @@ __device__ __forceinline__ bool carry_range(const FwdArgs& args, const void* in,
         if constexpr (!FIRONLY) {
             const long long sb = (lo + k) * B + sh - (T - 1);     // output spectrum of batch row 0
             static_for<NST>([&](auto p) {
-                fft_stage<C, B, NT, decltype(p)::value, OUT, S::TW_SMEM, S::SPW, false, false, S::LAYOUT, GRP, false, CONJ>(
-                    ybuf, tws, out, sb, vlo, vhi, nullptr, FREE ? &bars[NBAR - 1] : nullptr);
+                fft_stage<C, B, NT, decltype(p)::value, OUT, S::TW_SMEM, S::SPW, false, false, S::LAYOUT, GRP, CONJ>(
+                    ybuf, tws, out, sb, vlo, vhi, FREE ? &bars[NBAR - 1] : nullptr);
             });
         }
     }

@@ -209,17 +209,18 @@ struct RowShape {
     static constexpr bool TW_SMEM = RING ? fits(NR, true) : true;
     // 8/16-bit pairs are converted by two units (cvt_mixed); not with 16 taps held
     // in registers (C = 2048 T = 16: -1 %)
-    static constexpr bool MIXED = PAIR && IN != IN_CF32 && (L <= 5 || TM <= 8);
+    static constexpr bool MIXED = PAIR && IN != IN_CF32 && (L <= 5 || TM <= 8 || TM > 16);
     // STAGE: each thread copies the rows of its columns ahead of their use
     // with cp.async into NCH groups of GR slots of its own
     static constexpr int CB = BIN * (PAIR ? 2 : 1);                      // bytes of one copy
+    static constexpr int LW = PAIR && L > 8 ? L / 2 : L;                 // outputs at a time with many taps
     static constexpr int RW = L + TM - 1;                                // rows of a segment
     static constexpr int NROW = R0 * RW;                                 // copies per thread and batch
     static constexpr int GR = 2;
     static constexpr int NGR = (NROW + GR - 1) / GR;                     // groups per batch
     static constexpr int NCH0 = (CAP - YBYTES - TWBYTES - 64) / (GR * NT * CB);
     static constexpr int NCH1 = NCH0 > 8 ? 8 : NCH0;
-    static constexpr bool STAGE = !RING && IN == IN_CF32 && PAIR && R0 <= 3;
+    static constexpr bool STAGE = !RING && IN == IN_CF32 && PAIR && R0 <= 3 && TM <= 16;
     static constexpr int NCH = !STAGE ? 0 : NCH1 < NGR ? NCH1 : NGR;
     // batches ahead whose new rows are brought into L2: one where the rows that
     // all CTAs keep live stay within half of it (FP32 at C = 4096, T = 8: 75 MB
@@ -228,7 +229,7 @@ struct RowShape {
     static constexpr int RING_OFF = YBYTES + (TW_SMEM ? TWBYTES : 0);
     static constexpr int BAR_OFF = RING_OFF + NR * ROWB + NCH * GR * NT * CB;
     static constexpr int SMEM = BAR_OFF + 64;
-    static constexpr bool OK = TM <= 16 && SMEM <= CAP && (!STAGE || (CB >= 4 && NCH >= 2));
+    static constexpr bool OK = SMEM <= CAP && (!STAGE || (CB >= 4 && NCH >= 2));
     static_assert(B == L * G && RING_OFF % 16 == 0 && ROWB % 16 == 0, "whole segments, 16-byte aligned rows");
 };
 
@@ -429,7 +430,55 @@ __device__ __forceinline__ bool row_range(const FwdArgs& args, const void* in, v
                     accp[a][j] = 0ull;
                     if constexpr (PAIR) acci[a][j] = 0ull;
                 }
-                if constexpr (L <= 5) {
+                if constexpr (TM > 16) {
+                    // many taps (T is a runtime bound): taps outermost, a window of
+                    // LW rows in registers, LW outputs at a time.  Bound by the loads'
+                    // latency, hence the blocks: tap by tap C = 4096 int8 T = 64 took 23
+                    // GS/s, in blocks 56 (the generic kernel 14; C = 1024 int8 T = 32 168
+                    // against 90, C = 384 FP32 T = 64 95 against 45)
+                    constexpr int LW = S::LW;
+#pragma unroll
+                    for (int j0 = 0; j0 < L; j0 += LW) {
+                        u64 x0[LW], x1[LW];
+#pragma unroll
+                        for (int i = 0; i < LW; ++i) row(a, j0 + i, x0[i], x1[i]);
+                        auto fma_tap = [&](u64 h, int u) {
+#pragma unroll
+                            for (int j = 0; j < LW; ++j) {
+                                ffma2(accp[a][j0 + j], h, x0[(j + u) % LW]);
+                                if constexpr (PAIR) ffma2(acci[a][j0 + j], h, x1[(j + u) % LW]);
+                            }
+                        };
+                        int tb = 0;
+                        // whole blocks of taps without checks: their loads go out together
+                        auto block = [&](auto size_tag) {
+                            constexpr int N = decltype(size_tag)::value;
+                            u64 h[N];
+#pragma unroll
+                            for (int u = 0; u < N; ++u) h[u] = tap(a, tb + u);
+#pragma unroll
+                            for (int u = 0; u < N; ++u) {
+                                fma_tap(h[u], u);
+                                if (u + 1 < N || tb + N < T) row(a, j0 + tb + u + LW, x0[u % LW], x1[u % LW]);
+                            }
+                            tb += N;
+                        };
+                        constexpr int BLK = LW * ((8 + LW - 1) / LW);
+#pragma unroll 1
+                        while (tb + BLK <= T) block(ic<BLK>{});
+                        if constexpr (BLK > LW) {
+#pragma unroll 1
+                            while (tb + LW <= T) block(ic<LW>{});
+                        }
+#pragma unroll
+                        for (int u = 0; u < LW - 1; ++u) {
+                            if (tb + u < T) {
+                                fma_tap(tap(a, tb + u), u);
+                                if (tb + u + 1 < T) row(a, j0 + tb + u + LW, x0[u], x1[u]);
+                            }
+                        }
+                    }
+                } else if constexpr (L <= 5) {
                     // taps outermost, a window of L rows in registers
                     u64 x0[L], x1[L];
 #pragma unroll

@@ -1,7 +1,8 @@
 """The row kernel (large channel counts) at the sizes where it can go wrong:
 one output, ragged last batches, the edge between its small batches (calls
 that give an SM at most one) and its whole ones, ranges of several batches,
-tap counts below their bucket.  Tolerance: relative L2 <= 1e-5 against the
+tap counts below their bucket and, beyond 16 taps, around the blocks of its
+loop.  Tolerance: relative L2 <= 1e-5 against the
 FP64 oracle, as for every complex FP32 output; both batch sizes do the same
 arithmetic per output, so their results are equal bit for bit.
 """
@@ -19,7 +20,9 @@ ROW = 128                                             # plan_info variant bit of
 SHAPES = [(384, 8, "ci8"), (384, 13, "cf32"), (768, 3, "ci16"), (768, 16, "ci16"), (1024, 8, "ci16"), (1024, 5, "cf32"),
           (1024, 16, "ci8"), (1536, 7, "ci16"), (1536, 1, "cf32"), (2048, 8, "ci8"), (2048, 3, "cf32"),
           (2048, 16, "cf32"), (3072, 8, "ci16"), (3072, 6, "cf32"), (4096, 8, "ci8"), (4096, 13, "ci8"),
-          (4096, 2, "ci16"), (4096, 6, "cf32")]
+          (4096, 2, "ci16"), (4096, 6, "cf32"),
+          (384, 23, "ci8"), (384, 40, "cf32"), (768, 33, "ci16"), (1024, 20, "cf32"), (1024, 64, "ci8"), (1536, 17, "cf32"),
+          (2048, 31, "ci16"), (3072, 19, "cf32"), (3072, 64, "ci8"), (4096, 17, "ci8"), (4096, 45, "cf32")]
 
 
 @pytest.fixture(scope="module")
@@ -53,7 +56,7 @@ def test_short_and_long_calls_agree(ppf, C, T, in_dtype):
     assert oracle.rel_l2_max_per_spectrum(got, oracle.pfb_spectra(x, h, C, T, idx)) <= 1e-5
 
 
-@pytest.mark.parametrize("C,T", [(384, 5), (1024, 6), (1024, 3), (3072, 8), (4096, 3), (2048, 13)])
+@pytest.mark.parametrize("C,T", [(384, 5), (1024, 6), (1024, 3), (3072, 8), (4096, 3), (2048, 13), (1024, 21), (3072, 32), (4096, 18)])
 @pytest.mark.parametrize("bad", [np.inf, np.nan])
 def test_non_finite_sample_reaches_only_its_spectra(ppf, C, T, bad):
     """One inf or NaN sample of FP32 input reaches the T output spectra that read it and
