@@ -37,7 +37,7 @@
 // longer fit L2 and the halo is read from HBM again (C = 1536 FP32 T = 8: 1.77
 // instead of 1.07 GB read, 209 vs 266 GS/s).
 //
-// What bounds it: 57 instructions per sample at 40 % issue with 16 warps of
+// What bounds it: 64 instructions per sample (C = 4096 int8) at 48 % issue with 16 warps of
 // 128 registers; the FIR takes a quarter of the time, shared memory traffic
 // (about half of the LSU's rate) and the DFT the rest.  Against the generic
 // kernel it replaces (GS/s, 2^27 samples per launch, T = 8): C = 4096 int8 230 ->
@@ -434,8 +434,8 @@ __device__ __forceinline__ bool row_range(const FwdArgs& args, const void* in, v
                     // many taps (T is a runtime bound): taps outermost, a window of
                     // LW rows in registers, LW outputs at a time.  Bound by the loads'
                     // latency, hence the blocks: tap by tap C = 4096 int8 T = 64 took 23
-                    // GS/s, in blocks 56 (the generic kernel 14; C = 1024 int8 T = 32 168
-                    // against 90, C = 384 FP32 T = 64 95 against 45)
+                    // GS/s, in blocks 59 (the generic kernel 14; C = 1024 int8 T = 32 174
+                    // against 91, C = 384 FP32 T = 64 93 against 45)
                     constexpr int LW = S::LW;
 #pragma unroll
                     for (int j0 = 0; j0 < L; j0 += LW) {
