@@ -41,6 +41,11 @@
 
 namespace ppf {
 
+// Rows come as boxes of a tensor map of (channel, row, stream), whose strides have
+// to be multiples of one another.  Streams that lie no whole number of rows
+// apart have no such map: their rows are copied one by one.
+__host__ __device__ inline bool longtap_boxes(const FwdArgs& a, int C) { return a.n_streams == 1 || a.in_stride % C == 0; }
+
 // DIV = 1: batches of 32 outputs.  DIV = 2: of 16, for calls too short to give
 // every SM a batch of 32; the same arithmetic per output.
 template <int C, int IN, int DIV = 1>
@@ -57,7 +62,8 @@ struct LongShape {
     static constexpr int YBYTES = B * C * 8;
     static constexpr int TWBYTES = tw_size(C) * 8;
     static constexpr int TAPB = RC * NCT * 4;                        // a chunk: 8 taps, then 8 rows
-    static constexpr int CHUNKB = TAPB + RC * NCT * BIN;
+    static constexpr int ROWB = NCT * BIN;                           // one pass's channels of a row
+    static constexpr int CHUNKB = TAPB + RC * ROWB;
     static constexpr int RING_OFF = (YBYTES + TWBYTES + 127) / 128 * 128;
     static constexpr int CAP = (228 * 1024) / MINB - 1024 - 256;
     static constexpr int NS0 = (CAP - RING_OFF) / (CHUNKB + 16);
@@ -123,6 +129,7 @@ pfb_fwd_longtap_kernel(FwdArgs args, const __grid_constant__ CUtensorMap in_map,
 
     if (tid >= NCT) {
         // ------------------------------------------------ producer warp
+        const bool boxes = longtap_boxes(args, C);
         long long issued = 0;
         bool ok = true;
         while (ok && share.next(strm, lo, hi)) {
@@ -135,10 +142,22 @@ pfb_fwd_longtap_kernel(FwdArgs args, const __grid_constant__ CUtensorMap in_map,
                         const int t0 = (c - B / RC) * RC;            // the chunk's first tap
                         if (lane == 0) {
                             unsigned char* dst = ring + slot * S::CHUNKB;
+                            const long long r0 = k * B + c * RC;
+                            const uint32_t tapb = t0 >= 0 ? S::TAPB : 0;
                             fence_proxy_async_smem();
-                            mbar_expect_tx(&full[slot], t0 >= 0 ? S::CHUNKB : S::CHUNKB - S::TAPB);
-                            // rows past the stream are filled with zeros
-                            tma_load_box3(dst + S::TAPB, &in_map, p * NCT, (int)(k * B + c * RC), (int)strm, &full[slot]);
+                            if (boxes) {
+                                // rows past the stream are filled with zeros
+                                mbar_expect_tx(&full[slot], tapb + RC * S::ROWB);
+                                tma_load_box3(dst + S::TAPB, &in_map, p * NCT, (int)r0, (int)strm, &full[slot]);
+                            } else {
+                                // rows past the stream are left as they are: no stored output reads them
+                                const int rows = (int)(n_raw - r0 < 0 ? 0 : n_raw - r0 < RC ? n_raw - r0 : RC);
+                                const unsigned char* src = static_cast<const unsigned char*>(args.in) +
+                                                           (size_t)(strm * args.in_stride + r0 * C + p * NCT) * BIN;
+                                mbar_expect_tx(&full[slot], tapb + rows * S::ROWB);
+                                for (int i = 0; i < rows; ++i)
+                                    tma_load_1d(dst + S::TAPB + i * S::ROWB, src + (size_t)i * C * BIN, S::ROWB, &full[slot]);
+                            }
                             if (t0 >= 0) tma_load_box2(dst, &tap_map, p * NCT, t0, &full[slot]);
                         }
                         __syncwarp();
@@ -255,11 +274,13 @@ pfb_fwd_longtap_kernel(FwdArgs args, const __grid_constant__ CUtensorMap in_map,
 }
 
 // Tensor maps of a launch: the streams' samples as (channel, row, stream) in
-// boxes of 8 rows of NCT channels, and the plan's tap table (64 rows).
+// boxes of 8 rows of NCT channels (the first stream's only where the rows come
+// one by one), and the plan's tap table (64 rows).
 inline cudaError_t longtap_maps(const FwdArgs& a, int C, int bin, int nct, CUtensorMap* in_map, CUtensorMap* tap_map) {
     const unsigned long long n_raw = a.n_spectra + a.T - 1, row = (unsigned long long)C * bin;
-    const cudaError_t ce = make_tmap(in_map, a.in, bin, C, n_raw, row, a.n_streams,
-                                     a.n_streams > 1 ? a.in_stride * bin : n_raw * row, nct, 8);
+    const bool one = a.n_streams == 1 || !longtap_boxes(a, C);
+    const cudaError_t ce = make_tmap(in_map, a.in, bin, C, n_raw, row, one ? 1 : a.n_streams,
+                                     one ? n_raw * row : a.in_stride * bin, nct, 8);
     return ce != cudaSuccess ? ce : make_tmap(tap_map, a.taps, 4, C, 64, C * 4ull, 0, 0, nct, 8);
 }
 

@@ -15,7 +15,7 @@ inline CUtensorMapDataType tmap_type(int bytes) {
 // Rows of `cols` items of `bytes`, `rows` of them (row_bytes apart) in each of
 // `planes` planes (plane_bytes apart), in boxes of box_cols x box_rows of one
 // plane; planes = 0 makes the map two-dimensional.  Loads outside give zeros.
-// base and the strides are multiples of 16 bytes.
+// base and the strides are multiples of 16 bytes, plane_bytes of row_bytes.
 inline cudaError_t make_tmap(CUtensorMap* map, const void* base, int bytes, unsigned long long cols,
                              unsigned long long rows, unsigned long long row_bytes, unsigned long long planes,
                              unsigned long long plane_bytes, unsigned box_cols, unsigned box_rows) {
@@ -29,6 +29,7 @@ inline cudaError_t make_tmap(CUtensorMap* map, const void* base, int bytes, unsi
         return reinterpret_cast<Encode>(fn);
     }();
     if (encode == nullptr) return cudaErrorNotSupported;
+    if (row_bytes % 16 != 0 || (planes > 0 && plane_bytes % row_bytes != 0)) return cudaErrorInvalidValue;
     const cuuint64_t dims[3] = {cols, rows, planes}, strides[2] = {row_bytes, plane_bytes};
     const cuuint32_t box[3] = {box_cols, box_rows, 1}, one[3] = {1, 1, 1};
     return encode(map, tmap_type(bytes), planes > 0 ? 3 : 2, const_cast<void*>(base), dims, strides, box, one,
