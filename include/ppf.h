@@ -143,7 +143,9 @@ ppf_status ppf_execute_batched(ppf_plan_t plan, const void* in_dev, long long in
  * If a bounded device wait gives up (ppf_check_device then reports
  * PPF_ERR_DEVICE_TIMEOUT), grad_in is incomplete and every element of
  * grad_taps is NaN; the plan's status word stays set until ppf_check_device
- * clears it, and tap gradients computed meanwhile are NaN too.
+ * clears it, and tap gradients computed meanwhile are NaN too.  On the three-pass
+ * path so is grad_in where the word was set before its second pass (the inverse
+ * DFT gave up, or an earlier launch did): g_y cannot be relied on then.
  * Errors: INVALID_ARG, UNSUPPORTED, ALIGNMENT, CUDA, OUT_OF_MEMORY.
  */
 ppf_status ppf_backward(ppf_plan_t plan, const void* grad_out_dev, const void* in_dev, void* grad_in_dev,
@@ -303,7 +305,7 @@ ppf_status ppf_check_device(ppf_plan_t plan, ppf_stream_t stream);
  *   PPF_DEBUG_INJECT_TIMEOUT (1): every later launch of the plan's
  *     staged-input kernel waits on a barrier that nothing completes, so the
  *     bounded wait runs out (after 2 ms) and the timeout path is exercised
- *     without faulting the GPU;
+ *     without faulting the GPU (ppf_backward's kernels included);
  *   PPF_DEBUG_UNFUSED_ADJOINT (2): ppf_backward runs its three-pass path even
  *     where the fused adjoint kernel exists (to compare the two paths;
  *     ppf_backward_noalloc ignores it).

@@ -447,7 +447,7 @@ static ppf_status backward_unfused(ppf_plan_t p, const void* grad_out_dev, const
     ia.n_spectra = n_spectra;
     ia.n_streams = n_streams;
     ia.T = 1;
-    ia.flags = 0;
+    ia.flags = p->debug_flags;
     const ppf_status is = launch_entry(p->idft, p->idft_grid, p->sms, ia, "ppf_backward: inverse DFT launch", st);
     if (is != PPF_OK) return is;
     // parts of the row tiles of all streams, one CTA per part and channel block;
@@ -473,6 +473,7 @@ static ppf_status backward_unfused(ppf_plan_t p, const void* grad_out_dev, const
     ga.C = C;
     ga.T = T;
     ga.TM = TM;
+    ga.flags = p->debug_flags;
     ce = ppf::bwd_grad((int)p->in, ga, p->d_gy, in_dev, p->d_taps, (int)parts, st);
     if (ce != cudaSuccess) return cuda_fail(ce, "ppf_backward: gradient launch");
     if (grad_taps_dev != nullptr) {

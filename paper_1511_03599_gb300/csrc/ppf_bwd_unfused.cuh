@@ -98,6 +98,7 @@ struct AdjArgs {
     int* err;
     long long n_spectra, n_streams;
     int C, T, TM;
+    int flags;               // FwdFlags (testing aid)
 };
 
 struct AdjMaps {
@@ -128,6 +129,7 @@ pfb_bwd_grad_kernel(AdjArgs a, const __grid_constant__ CUtensorMap g_map, const 
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + S::BAR_OFF);     // [NS] chunk landed
     uint64_t* empty = full + NS;                                          // [NS] every consumer warp is done with it
     volatile int* sdead = reinterpret_cast<volatile int*>(full + 2 * NS);
+    uint64_t* inj = full + 2 * NS + 1;                                    // never completed (testing aid)
     float* ghs = reinterpret_cast<float*>(smem + S::GH_OFF);              // [T][NCT]
 
     grid_dependency_wait();                                               // launched by launch_early
@@ -142,15 +144,29 @@ pfb_bwd_grad_kernel(AdjArgs a, const __grid_constant__ CUtensorMap g_map, const 
             mbar_init(&full[i], 1);
             mbar_init(&empty[i], NCT / 32);
         }
+        mbar_init(inj, 1);
         fence_mbar_init();
         *sdead = 0;
     }
     if (GH && tid < NCT)
         for (int t = 0; t < T; ++t) ghs[t * NCT + tid] = 0.f;
-    __syncthreads();
+    // the status word is set: the inverse DFT (or an earlier launch) gave up, g_y
+    // may not have been written
+    const bool failed = __syncthreads_or(tid == 0 && *static_cast<volatile int*>(a.err) != 0);
 
     BatchShare share(tiles, a.n_streams, blockIdx.x, gridDim.x);
     long long strm, lo, hi;
+    if (failed) {            // grad_x becomes NaN, as grad_h does in the reduction
+        if (GX && tid < NCT) {
+            const float nan = __int_as_float(0x7fc00000);
+            while (share.next(strm, lo, hi)) {
+                float2* out = a.gx + (size_t)strm * n_raw * a.C + c0 + tid;
+                const long long end = hi * L < n_raw ? hi * L : n_raw;
+                for (long long r = lo * L; r < end; ++r) out[(size_t)r * a.C] = make_float2(nan, nan);
+            }
+        }
+        return;
+    }
     // chunk use g sits in slot g mod NS and completes phase g / NS of its barriers
     int slot = 0;
     uint32_t phase = 0;
@@ -215,6 +231,10 @@ pfb_bwd_grad_kernel(AdjArgs a, const __grid_constant__ CUtensorMap g_map, const 
         if (lane == 0) mbar_arrive_cta(&empty[slot]);
         advance();
     };
+    if (tid == 0 && (a.flags & FWD_INJECT_TIMEOUT) && !mbar_wait_bounded(inj, 0, kInjectedWaitNs)) {
+        atomicExch(a.err, 1);
+        *sdead = 1;
+    }
     while (share.next(strm, lo, hi)) {
         for (long long k = lo; k < hi; ++k) {
             const long long r0 = k * L;

@@ -1,0 +1,53 @@
+"""A bounded device wait that runs out (a barrier that nothing completes, 2 ms) in
+the kernels of the three-pass adjoint: the status is reported, no gradient looks
+complete, and the next call is right.  At C >= 64 the inverse DFT gives up and the
+second pass must not use its rows; at C = 32, whose inverse DFT waits for
+nothing, the second pass gives up itself.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1511_03599_gb300 import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+SIGMA = {"ci8": 16.0, "ci16": 2000.0, "cf32": 1.0}
+
+
+@pytest.fixture(scope="module")
+def ppf():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1511_03599_gb300 import ppf as m
+    m.lib()
+    return m
+
+
+@pytest.mark.parametrize("C,T,in_dtype,S", [(512, 32, "ci8", 20), (512, 32, "ci8", 900), (512, 16, "cf32", 5000),
+                                            (1024, 8, "cf32", 300), (4096, 8, "ci8", 40), (3072, 3, "ci16", 150),
+                                            (128, 17, "ci16", 2500), (32, 8, "cf32", 3000)])
+def test_three_pass_adjoint_reports_a_timeout(ppf, C, T, in_dtype, S):
+    rng = np.random.default_rng(C + T)
+    h = synth.design_taps(C, T)
+    x = synth.stream(C, S + T - 1, in_dtype, SIGMA[in_dtype], 9500 + C)
+    xd = torch.from_numpy(x).cuda()
+    G = torch.from_numpy((rng.standard_normal((S, C)) + 1j * rng.standard_normal((S, C))).astype(np.complex64)).cuda()
+    with ppf.Plan(C, T, h, in_dtype, "c64") as plan:
+        plan.set_debug_flags(1)
+        for want_input, want_taps in ((True, True), (True, False), (False, True)):
+            gx, gh = plan.backward(G, xd, want_input=want_input, want_taps=want_taps)
+            with pytest.raises(ppf.PPFError) as ei:
+                plan.check_device()
+            assert ei.value.status == 5
+            if want_input and C != 32:
+                assert bool(torch.isnan(torch.view_as_real(gx)).all())
+            if want_taps:
+                assert bool(torch.isnan(gh).all())
+        plan.set_debug_flags(0)
+        gx, gh = plan.backward(G, xd)
+        plan.check_device()
+    Gn = G.cpu().numpy().astype(np.complex128)
+    assert oracle.rel_l2(gx.cpu().numpy().reshape(-1), oracle.pfb_grad_input(Gn, h, C, T).reshape(-1)) <= 1e-5
+    assert oracle.rel_l2(gh.cpu().numpy(), oracle.pfb_grad_taps(Gn, x, C, T)) <= 1e-4
