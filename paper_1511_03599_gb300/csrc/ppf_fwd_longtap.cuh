@@ -43,8 +43,9 @@ namespace ppf {
 
 // Rows come as boxes of a tensor map of (channel, row, stream), whose strides have
 // to be multiples of one another.  Streams that lie no whole number of rows
-// apart have no such map: their rows are copied one by one.
-__host__ __device__ inline bool longtap_boxes(const FwdArgs& a, int C) { return a.n_streams == 1 || a.in_stride % C == 0; }
+// apart have no such map: their rows are copied one by one (ROWS, a form of its
+// own: beside the boxes in one kernel it cost 1.5 % at C = 512, T = 64, FP32).
+inline bool longtap_boxes(const FwdArgs& a, int C) { return a.n_streams == 1 || a.in_stride % C == 0; }
 
 // DIV = 1: batches of 32 outputs.  DIV = 2: of 16, for calls too short to give
 // every SM a batch of 32; the same arithmetic per output.
@@ -74,7 +75,7 @@ struct LongShape {
                                NS >= 3 && SMEM <= CAP;
 };
 
-template <int C, int IN, int OUT, int DIV = 1>
+template <int C, int IN, int OUT, int DIV = 1, bool ROWS = false>
 __global__ void __launch_bounds__(LongShape<C, IN, DIV>::NT, LongShape<C, IN, DIV>::MINB)
 pfb_fwd_longtap_kernel(FwdArgs args, const __grid_constant__ CUtensorMap in_map, const __grid_constant__ CUtensorMap tap_map) {
     using S = LongShape<C, IN, DIV>;
@@ -92,7 +93,7 @@ pfb_fwd_longtap_kernel(FwdArgs args, const __grid_constant__ CUtensorMap in_map,
     uint64_t* inj = full + 2 * NS;                                       // never completed (testing aid)
     volatile int* sdead = reinterpret_cast<volatile int*>(full + 2 * NS + 1);
 
-    if constexpr (DIV > 1) grid_dependency_wait();   // launched by launch_early
+    if constexpr (DIV > 1 || ROWS) grid_dependency_wait();   // launched by launch_early
     const int tid = threadIdx.x, lane = tid & 31;
     const long long n_spectra = args.n_spectra;
     const int T = args.T;                        // 17 .. 64
@@ -129,7 +130,6 @@ pfb_fwd_longtap_kernel(FwdArgs args, const __grid_constant__ CUtensorMap in_map,
 
     if (tid >= NCT) {
         // ------------------------------------------------ producer warp
-        const bool boxes = longtap_boxes(args, C);
         long long issued = 0;
         bool ok = true;
         while (ok && share.next(strm, lo, hi)) {
@@ -140,23 +140,27 @@ pfb_fwd_longtap_kernel(FwdArgs args, const __grid_constant__ CUtensorMap in_map,
                         ok = __all_sync(0xffffffffu, ok);
                         if (!ok) break;
                         const int t0 = (c - B / RC) * RC;            // the chunk's first tap
+                        unsigned char* dst = ring + slot * S::CHUNKB;
+                        if constexpr (ROWS) {
+                            // a row per lane; rows past the stream are left as they are: no stored output reads them
+                            const long long r = k * B + c * RC, left = n_raw - r;
+                            const int rows = left < 0 ? 0 : left < RC ? (int)left : RC;
+                            if (lane == 0) mbar_expect_tx(&full[slot], (t0 >= 0 ? S::TAPB : 0) + rows * S::ROWB);
+                            __syncwarp();
+                            if (lane < rows) {
+                                fence_proxy_async_smem();
+                                tma_load_1d(dst + S::TAPB + lane * S::ROWB,
+                                            static_cast<const unsigned char*>(args.in) +
+                                                (size_t)(strm * args.in_stride + (r + lane) * C + p * NCT) * BIN,
+                                            S::ROWB, &full[slot]);
+                            }
+                        }
                         if (lane == 0) {
-                            unsigned char* dst = ring + slot * S::CHUNKB;
-                            const long long r0 = k * B + c * RC;
-                            const uint32_t tapb = t0 >= 0 ? S::TAPB : 0;
                             fence_proxy_async_smem();
-                            if (boxes) {
+                            if constexpr (!ROWS) {
+                                mbar_expect_tx(&full[slot], t0 >= 0 ? S::CHUNKB : S::CHUNKB - S::TAPB);
                                 // rows past the stream are filled with zeros
-                                mbar_expect_tx(&full[slot], tapb + RC * S::ROWB);
-                                tma_load_box3(dst + S::TAPB, &in_map, p * NCT, (int)r0, (int)strm, &full[slot]);
-                            } else {
-                                // rows past the stream are left as they are: no stored output reads them
-                                const int rows = (int)(n_raw - r0 < 0 ? 0 : n_raw - r0 < RC ? n_raw - r0 : RC);
-                                const unsigned char* src = static_cast<const unsigned char*>(args.in) +
-                                                           (size_t)(strm * args.in_stride + r0 * C + p * NCT) * BIN;
-                                mbar_expect_tx(&full[slot], tapb + rows * S::ROWB);
-                                for (int i = 0; i < rows; ++i)
-                                    tma_load_1d(dst + S::TAPB + i * S::ROWB, src + (size_t)i * C * BIN, S::ROWB, &full[slot]);
+                                tma_load_box3(dst + S::TAPB, &in_map, p * NCT, (int)(k * B + c * RC), (int)strm, &full[slot]);
                             }
                             if (t0 >= 0) tma_load_box2(dst, &tap_map, p * NCT, t0, &full[slot]);
                         }
@@ -288,8 +292,13 @@ template <int C, int IN, int OUT, int DIV>
 inline cudaError_t longtap_launch(const FwdArgs& a, int grid, cudaStream_t st) {
     using S = LongShape<C, IN, DIV>;
     CUtensorMap in_map, tap_map;
-    const cudaError_t ce = longtap_maps(a, C, S::BIN, S::NCT, &in_map, &tap_map);
+    cudaError_t ce = longtap_maps(a, C, S::BIN, S::NCT, &in_map, &tap_map);
     if (ce != cudaSuccess) return ce;
+    if (!longtap_boxes(a, C)) {
+        constexpr auto k = &pfb_fwd_longtap_kernel<C, IN, OUT, DIV, true>;
+        ce = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, S::SMEM);
+        return ce != cudaSuccess ? ce : launch_early(k, grid, S::NT, S::SMEM, st, a, in_map, tap_map);
+    }
     if constexpr (DIV > 1) {
         return launch_early(pfb_fwd_longtap_kernel<C, IN, OUT, DIV>, grid, S::NT, S::SMEM, st, a, in_map, tap_map);
     } else {
