@@ -183,7 +183,7 @@ pfb_bwd_grad_kernel(AdjArgs a, const __grid_constant__ CUtensorMap g_map, const 
         while (ok && share.next(strm, lo, hi)) {
             for (long long k = lo; ok && k < hi; ++k) {
                 for (int c = 0; c < nch; ++c) {
-                    if (issued >= NS) ok = !*sdead && mbar_wait_bounded(&empty[slot], phase ^ 1, kWaitLimitNs);
+                    if (issued >= NS) ok = mbar_wait_bounded_or(&empty[slot], phase ^ 1, kWaitLimitNs, sdead);
                     ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
                     if (lane == 0) {
@@ -304,13 +304,14 @@ pfb_bwd_grad_kernel(AdjArgs a, const __grid_constant__ CUtensorMap g_map, const 
             };
             if (GH && IN == IN_CF32 && (r0 < T - 1 || r0 + L > a.n_spectra)) steps(ic<1>{});
             else steps(ic<0>{});
+            // a wait gave up: this warp stores nothing more (the producer and the
+            // other warps leave the same way)
+            if (__any_sync(0xffffffffu, *sdead != 0)) return;
             if constexpr (GX) {
-                if (!*sdead) {
-                    float2* out = a.gx + ((size_t)strm * n_raw + r0) * a.C + c0 + tid;
+                float2* out = a.gx + ((size_t)strm * n_raw + r0) * a.C + c0 + tid;
 #pragma unroll
-                    for (int j = 0; j < L; ++j)
-                        if (r0 + j < n_raw) __stcs(out + (size_t)j * a.C, upk2(acc[j]));
-                }
+                for (int j = 0; j < L; ++j)
+                    if (r0 + j < n_raw) __stcs(out + (size_t)j * a.C, upk2(acc[j]));
             }
         }
     }

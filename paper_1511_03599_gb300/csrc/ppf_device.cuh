@@ -335,6 +335,18 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
     }
     return true;
 }
+// The same, giving up as well once *stop is set (also by a thread that set it
+// and then arrived on the barrier).
+__device__ __forceinline__ bool mbar_wait_bounded_or(uint64_t* bar, uint32_t parity, uint64_t limit_ns,
+                                                     const volatile int* stop) {
+    if (!mbar_try_wait(bar, parity)) {
+        const uint64_t t0 = globaltimer_ns();
+        while (!mbar_try_wait(bar, parity)) {
+            if (*stop || globaltimer_ns() - t0 > limit_ns) return false;
+        }
+    }
+    return !*stop;
+}
 // 1-D bulk copy global -> shared completing on `bar` (bytes multiple of 16,
 // both addresses 16-byte aligned).
 __device__ __forceinline__ void tma_load_1d(void* dst_smem, const void* src_gmem, uint32_t bytes, uint64_t* bar) {

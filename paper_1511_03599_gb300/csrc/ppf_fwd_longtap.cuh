@@ -91,7 +91,8 @@ pfb_fwd_longtap_kernel(FwdArgs args, const __grid_constant__ CUtensorMap in_map,
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + S::BAR_OFF);    // [NS] chunk landed
     uint64_t* empty = full + NS;                                         // [NS] every consumer warp is done with it
     uint64_t* inj = full + 2 * NS;                                       // never completed (testing aid)
-    volatile int* sdead = reinterpret_cast<volatile int*>(full + 2 * NS + 1);
+    volatile int* sdead = reinterpret_cast<volatile int*>(full + 2 * NS + 1);   // a wait gave up
+    volatile int* sgone = sdead + 1;                                     // what the consumers go by: one value a batch
 
     if constexpr (DIV > 1 || ROWS) grid_dependency_wait();   // launched by launch_early
     const int tid = threadIdx.x, lane = tid & 31;
@@ -136,7 +137,7 @@ pfb_fwd_longtap_kernel(FwdArgs args, const __grid_constant__ CUtensorMap in_map,
             for (long long k = lo; ok && k < hi; ++k) {
                 for (int p = 0; ok && p < NPASS; ++p) {
                     for (int c = 0; c < nch; ++c) {
-                        if (issued >= NS) ok = !*sdead && mbar_wait_bounded(&empty[slot], phase ^ 1, kWaitLimitNs);
+                        if (issued >= NS) ok = mbar_wait_bounded_or(&empty[slot], phase ^ 1, kWaitLimitNs, sdead);
                         ok = __all_sync(0xffffffffu, ok);
                         if (!ok) break;
                         const int t0 = (c - B / RC) * RC;            // the chunk's first tap
@@ -263,9 +264,16 @@ pfb_fwd_longtap_kernel(FwdArgs args, const __grid_constant__ CUtensorMap in_map,
 #pragma unroll
                 for (int j = 0; j < B; ++j) ybuf[j * C + p * NCT + tid] = upk2(acc[j]);
             }
+            if (tid == 0) *sgone = *sdead;
             sync();
+            // A CTA that gave up stores nothing and leaves, with the producer: before the
+            // DFT at C = 512, after it elsewhere, where each left the kernel as fast
+            // as without the exit (the other way -1.8 % at C = 512, T = 64, FP32, and
+            // -3 % at C = 128, T = 17, through code generation)
+            const bool gone = *sgone != 0;
+            if (NPASS > 1 && gone) return;
             // ------------------------------------------------------- FFT
-            const long long vhi = *sdead ? 0 : n_spectra;            // a CTA that gave up stores nothing
+            const long long vhi = NPASS == 1 && gone ? 0 : n_spectra;
 #pragma unroll 1
             for (int q = 0; q < B / 16; ++q) {
                 static_for<NST>([&](auto st) {
@@ -273,6 +281,7 @@ pfb_fwd_longtap_kernel(FwdArgs args, const __grid_constant__ CUtensorMap in_map,
                                                                                   k * B + q * 16, 0, vhi);
                 });
             }
+            if (NPASS == 1 && vhi == 0) return;
         }
     }
 }

@@ -51,3 +51,34 @@ def test_three_pass_adjoint_reports_a_timeout(ppf, C, T, in_dtype, S):
     Gn = G.cpu().numpy().astype(np.complex128)
     assert oracle.rel_l2(gx.cpu().numpy().reshape(-1), oracle.pfb_grad_input(Gn, h, C, T).reshape(-1)) <= 1e-5
     assert oracle.rel_l2(gh.cpu().numpy(), oracle.pfb_grad_taps(Gn, x, C, T)) <= 1e-4
+
+
+def _milliseconds(fn):
+    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    torch.cuda.synchronize()
+    a.record()
+    fn()
+    b.record()
+    torch.cuda.synchronize()
+    return a.elapsed_time(b)
+
+
+@pytest.mark.parametrize("C,T,in_dtype,S,back", [(64, 40, "ci8", 800000, False), (512, 40, "cf32", 60000, False),
+                                                 (32, 32, "cf32", 800000, True)])
+def test_a_launch_that_gave_up_ends_at_once(ppf, C, T, in_dtype, S, back):
+    """The time to leave does not grow with the batches left (the long-tap kernel and
+    the three-pass adjoint's second pass, dozens of batches per CTA): the 2 ms wait
+    and at most the batch at hand."""
+    dtype = {"ci8": torch.int8, "cf32": torch.float32}[in_dtype]
+    x = torch.ones((C * (S + T - 1), 2), dtype=dtype, device="cuda")
+    with ppf.Plan(C, T, synth.design_taps(C, T), in_dtype, "c64") as plan:
+        y = plan(x)
+        call = (lambda: plan.backward(y, x)) if back else (lambda: plan.execute(x, out=y))
+        call()
+        plan.check_device()
+        good = _milliseconds(call)
+        plan.set_debug_flags(1)
+        ms = _milliseconds(call)
+        with pytest.raises(ppf.PPFError):
+            plan.check_device()
+        assert 1.5 <= ms <= good + 30.0
