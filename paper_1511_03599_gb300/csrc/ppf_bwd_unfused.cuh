@@ -81,7 +81,8 @@ __global__ void __launch_bounds__(IdftShape<C>::NT) pfb_bwd_idft_kernel(FwdArgs 
 // written out once per CTA (partial sums, reduced in a fixed order later).
 // A producer warp keeps a ring of chunks filled with boxes of tensor maps: 8
 // rows of g_y with 8 rows of x (the window and the tile's samples), then 8
-// rows of g_y with 8 taps.  Rows outside a stream read as zeros.
+// rows of g_y with 8 taps.  Rows outside a stream read as zeros; ENDS, the form for
+// short streams, leaves out the steps that see nothing else (AdjSteps).
 // Bound by FP32 issue (2 T packed FMAs per sample, 1.0 clock per sample and SM at
 // T = 32; it takes 2.2, 52 % of the FMA pipe) and for few taps by HBM.  The two
 // kernels it replaces read g_y once each, the halo five times from L2 (tiles
@@ -101,6 +102,16 @@ struct AdjArgs {
     int flags;               // FwdFlags (testing aid)
 };
 
+// ENDS: the steps of the tile at raw row r0 are taps t1, t1 - 1, .., n of them, whose
+// window r0 - t .. r0 - t + kAdjL-1 meets rows 0 .. S-1 of the stream (at least one does).
+struct AdjSteps {
+    int t1, n;
+    __device__ __forceinline__ AdjSteps(long long r0, long long S, int T) {
+        t1 = r0 + kAdjL < T ? (int)r0 + kAdjL - 1 : T - 1;
+        n = t1 + 1 - (r0 >= S ? (int)(r0 - S) + 1 : 0);
+    }
+};
+
 struct AdjMaps {
     CUtensorMap g, x, taps;
 };
@@ -118,7 +129,7 @@ struct AdjShape {
     static constexpr int smem(int T) { return GH_OFF + T * NCT * 4; }
 };
 
-template <int IN, int NCT, bool GX, bool GH>
+template <int IN, int NCT, bool GX, bool GH, bool ENDS>
 __global__ void __launch_bounds__(AdjShape<IN, NCT>::NT, AdjShape<IN, NCT>::MINB)
 pfb_bwd_grad_kernel(AdjArgs a, const __grid_constant__ CUtensorMap g_map, const __grid_constant__ CUtensorMap x_map,
                     const __grid_constant__ CUtensorMap tap_map) {
@@ -138,7 +149,7 @@ pfb_bwd_grad_kernel(AdjArgs a, const __grid_constant__ CUtensorMap g_map, const 
     const int T = a.T;
     const long long n_raw = a.n_spectra + T - 1;
     const long long tiles = (n_raw + L - 1) / L;
-    const int nch = L / RC + (T + RC - 1) / RC;
+    int nch = L / RC + (T + RC - 1) / RC;
     if (tid == 0) {
         for (int i = 0; i < NS; ++i) {
             mbar_init(&full[i], 1);
@@ -182,6 +193,12 @@ pfb_bwd_grad_kernel(AdjArgs a, const __grid_constant__ CUtensorMap g_map, const 
         bool ok = true;
         while (ok && share.next(strm, lo, hi)) {
             for (long long k = lo; ok && k < hi; ++k) {
+                int t1 = T - 1;
+                if constexpr (ENDS) {
+                    const AdjSteps st(k * L, a.n_spectra, T);
+                    t1 = st.t1;
+                    nch = L / RC + (st.n + RC - 1) / RC;
+                }
                 for (int c = 0; c < nch; ++c) {
                     if (issued >= NS) ok = mbar_wait_bounded_or(&empty[slot], phase ^ 1, kWaitLimitNs, sdead);
                     ok = __all_sync(0xffffffffu, ok);
@@ -192,8 +209,8 @@ pfb_bwd_grad_kernel(AdjArgs a, const __grid_constant__ CUtensorMap g_map, const 
                         const int u = (c - L / RC) * RC;             // the chunk's first step
                         const bool first = u < 0;
                         mbar_expect_tx(&full[slot], S::GB + (first ? (GH ? RC * NCT * BIN : 0) : RC * NCT * 4));
-                        tma_load_box3(dst, &g_map, c0, (int)(k * L) - (T - 1) + c * RC, (int)strm, &full[slot]);
-                        if (!first) tma_load_box2(dst + S::GB, &tap_map, c0, T - RC - u, &full[slot]);
+                        tma_load_box3(dst, &g_map, c0, (int)(k * L) - t1 + c * RC, (int)strm, &full[slot]);
+                        if (!first) tma_load_box2(dst + S::GB, &tap_map, c0, t1 + 1 - RC - u, &full[slot]);
                         else if (GH) tma_load_box3(dst + S::GB, &x_map, c0, (int)(k * L) + c * RC, (int)strm, &full[slot]);
                     }
                     __syncwarp();
@@ -259,22 +276,28 @@ pfb_bwd_grad_kernel(AdjArgs a, const __grid_constant__ CUtensorMap g_map, const 
                 }
                 release();
             }
+            int t1 = T - 1, n = T;
+            if constexpr (ENDS) {
+                const AdjSteps st(r0, a.n_spectra, T);
+                t1 = st.t1;
+                n = st.n;
+            }
             auto steps = [&](auto edge_tag) {
-                // EDGE (FP32 input): some rows lie outside the stream; their zeros must
-                // not meet an inf or NaN sample
-                constexpr bool EDGE = decltype(edge_tag)::value != 0;
+                // EDGE (FP32 input): some rows lie outside the stream, and an inf or NaN
+                // sample must not meet their zeros
+                [[maybe_unused]] constexpr bool EDGE = decltype(edge_tag)::value != 0;
 #pragma unroll 1
-                for (int tb = 0; tb < T; tb += L) {
+                for (int tb = 0; tb < n; tb += L) {
 #pragma unroll
                     for (int blk = 0; blk < L / RC; ++blk) {
                         const int u0 = tb + blk * RC;
-                        if (u0 >= T) break;
+                        if (u0 >= n) break;
                         wait_full();
 #pragma unroll
                         for (int i = 0; i < RC; ++i) {
                             const int w = blk * RC + i;              // window slot of the oldest row
-                            const int t = T - 1 - u0 - i;
-                            if (t < 0) break;
+                            const int t = t1 - u0 - i;
+                            if (ENDS ? u0 + i >= n : t < 0) break;
                             if constexpr (GX) {
                                 const float hv = *reinterpret_cast<const float*>(smem + slot * S::CHUNKB + S::GB +
                                                                                  ((RC - 1 - i) * NCT + tid) * 4);
@@ -287,7 +310,10 @@ pfb_bwd_grad_kernel(AdjArgs a, const __grid_constant__ CUtensorMap g_map, const 
 #pragma unroll
                                 for (int j = 0; j < L; ++j) {
                                     u64 x = xs[j];
-                                    if constexpr (EDGE) {
+                                    if constexpr (EDGE && NCT < 128) {
+                                        // (a stream of 2^31 rows would not fit the device)
+                                        if ((unsigned)((int)r0 - t + j) >= (unsigned)a.n_spectra) continue;
+                                    } else if constexpr (EDGE) {
                                         const long long s = r0 + j - t;
                                         if (s < 0 || s >= a.n_spectra) x = 0ull;
                                     }
@@ -302,7 +328,25 @@ pfb_bwd_grad_kernel(AdjArgs a, const __grid_constant__ CUtensorMap g_map, const 
                     }
                 }
             };
-            if (GH && IN == IN_CF32 && (r0 < T - 1 || r0 + L > a.n_spectra)) steps(ic<1>{});
+            // EDGE's checks make a tile two to six times as long, so with 128 channels
+            // they wait for an inf or NaN sample at the ends of a stream (with fewer the
+            // search cost as much: C = 32, T = 8 -2 %)
+            bool odd = false;
+            if constexpr (GH && IN == IN_CF32) {
+                odd = r0 < T - 1 || r0 + L > a.n_spectra;
+                if constexpr (NCT == 128) {
+                    if (odd) {
+                        odd = false;
+#pragma unroll
+                        for (int j = 0; j < L; ++j) {
+                            const float2 v = upk2(xs[j]);
+                            odd |= !(fabsf(v.x) < INFINITY) | !(fabsf(v.y) < INFINITY);
+                        }
+                        odd = __any_sync(0xffffffffu, odd);
+                    }
+                }
+            }
+            if (GH && IN == IN_CF32 && odd) steps(ic<1>{});
             else steps(ic<0>{});
             // a wait gave up: this warp stores nothing more (the producer and the
             // other warps leave the same way)
