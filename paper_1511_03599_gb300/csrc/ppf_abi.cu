@@ -440,12 +440,15 @@ static ppf_status backward_unfused(ppf_plan_t p, const void* grad_out_dev, const
     ppf::FwdArgs ia;
     ia.in = grad_out_dev;
     ia.out = p->d_gy;
-    ia.in_stride = ia.out_stride = n_spectra * C;
+    ia.in_stride = ia.out_stride = 0;
     ia.taps = p->d_ones;
     ia.tw = p->d_tw;
     ia.err = p->d_err;
-    ia.n_spectra = n_spectra;
-    ia.n_streams = n_streams;
+    // with one tap the rows of all streams, which lie one after the other, are one
+    // stream: streams of a few rows then fill the batches (C = 1024 T = 1, 640 streams
+    // of 9 spectra: grad_in 62 -> 50 us)
+    ia.n_spectra = n_streams * n_spectra;
+    ia.n_streams = 1;
     ia.T = 1;
     ia.flags = p->debug_flags;
     const ppf_status is = launch_entry(p->idft, p->idft_grid, p->sms, ia, "ppf_backward: inverse DFT launch", st);

@@ -63,3 +63,22 @@ def test_non_finite_sample_at_the_ends(ppf, C, T, S, bad):
                     want[t, c] = False
             assert torch.equal(finite, want), r
             assert bool(torch.isfinite(torch.view_as_real(gx)).all())
+
+
+@pytest.mark.parametrize("C,T,S,ns", [(384, 4, 9, 300), (1024, 1, 3, 500), (512, 24, 5, 200), (32, 2, 7, 900)])
+def test_many_short_streams(ppf, C, T, S, ns):
+    """One inverse DFT over the rows of all streams: each stream's input gradient is, bit
+    for bit, the one of the stream alone, and the tap gradient the sum over the streams."""
+    rng = np.random.default_rng(C + ns)
+    h = synth.design_taps(C, T)
+    x = rng.integers(-50, 50, (ns, C * (S + T - 1), 2), dtype=np.int8)
+    G = (rng.standard_normal((ns, S, C)) + 1j * rng.standard_normal((ns, S, C))).astype(np.complex64)
+    xd, Gd = torch.from_numpy(x).cuda(), torch.from_numpy(G).cuda()
+    with ppf.Plan(C, T, h, "ci8", "c64") as plan:
+        gx, gh = plan.backward(Gd, xd)
+        for i in (0, 1, ns // 2, ns - 1):
+            alone, _ = plan.backward(Gd[i].clone(), xd[i].clone())
+            assert torch.equal(torch.view_as_real(gx[i]), torch.view_as_real(alone)), i
+        plan.check_device()
+    ref = sum(oracle.pfb_grad_taps(G[i].astype(np.complex128), x[i], C, T) for i in range(ns))
+    assert oracle.rel_l2(gh.cpu().numpy(), ref.reshape(-1)) <= 1e-4
