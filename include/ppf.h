@@ -196,7 +196,8 @@ ppf_status ppf_update_taps(ppf_plan_t plan, const float* taps_dev, ppf_stream_t 
  *   in [64, 4096]), T[i] <= 16 taps, n_spectra[i] output spectra and taps_host[i]
  *   (C[i]*T[i] FP32, tap-major; read during the call).  Complex int8 input and
  *   complex FP32 output only (else UNSUPPORTED).  The plan cuts every beam
- *   into tiles of about 2^13 to 2^20 samples (about 24 per SM), sorts them largest first into a wide
+ *   into equal tiles of at most about 2^13 to 2^20 samples (the size with which
+ *   the SMs are expected to end soonest), sorts them longest first into a wide
  *   (C >= 1024) and a narrow queue and keeps taps, twiddles, descriptors,
  *   tiles, two work-queue counters and a status word in device memory it
  *   allocates.  Synchronous.
@@ -211,11 +212,12 @@ ppf_status ppf_update_taps(ppf_plan_t plan, const float* taps_dev, ppf_stream_t 
  *   Each CTA first pulls wide tiles (beams with C >= 1024) and runs each with
  *   all its threads, then splits into two groups of 256 threads that pull
  *   narrow tiles (C <= 512) independently.  A tile runs the FIR + DFT body of
- *   a single-stream kernel: the carry kernel's at C = 1024 (FIR halo carried
- *   in registers), the row kernel's at C = 2048 and 4096, the generic kernel's
- *   otherwise (raw rows staged through a TMA ring).  Every beam's result equals ppf_execute's up to FP32 rounding
- *   (bit-identical at C = 1024 with up to 8 taps and at C = 4096, where
- *   ppf_execute runs the same body).  Asynchronous on `stream`; no allocation.
+ *   a single-stream kernel: the carry kernel's at C = 1024 with up to 8 taps
+ *   (FIR halo carried in registers), the row kernel's for the rest of C >= 1024,
+ *   the generic kernel's otherwise (raw rows staged through a TMA ring).  Every
+ *   beam's result equals ppf_execute's up to FP32 rounding (bit-identical at
+ *   C >= 1024, where ppf_execute runs the same body).  Asynchronous on `stream`;
+ *   no allocation.
  * ppf_beams_info -- info[0]=beams, [1]=tiles, [2]=tile samples, [3]=CTAs per SM,
  *   [4]=SMs, [5]=dynamic shared memory bytes, [6]=wide tiles (C >= 1024).
  * ppf_beams_check_device -- as ppf_check_device, for the multi-beam launch.

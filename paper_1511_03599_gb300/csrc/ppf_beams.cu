@@ -2,16 +2,17 @@
 // spectrum counts in ONE persistent launch.
 //
 // The plan cuts every beam into tiles (contiguous ranges of output batches of
-// about `tile_samples` samples: 2^13 to 2^20, by the size of the set) and sorts the tiles largest first in two
-// queues: beams with C >= 1024 ("wide" tiles) and beams with C <= 512
+// at most about `tile_samples` samples: 2^13 to 2^20, pick_tile_samples) and
+// sorts the tiles longest first in two queues: beams with C >= 1024 ("wide" tiles) and beams with C <= 512
 // ("narrow" tiles).  The grid is persistent: one CTA of 512 threads per SM.
 // Each CTA first pulls wide tiles from a device counter and runs each with
-// the whole CTA: at C = 1024 the body of the carry kernel (one channel pair
-// per thread, the FIR halo carried in registers, warp-local DFT stages), at
-// C >= 2048 the body of the row kernel (first DFT stage on the FIR's registers).  When the wide queue is empty, the CTA splits into two
-// groups of 256 threads, each with half of the shared memory and its own
-// named barrier, and each group pulls narrow tiles from the second counter
-// and runs them independently with the generic body.
+// the whole CTA: at C = 1024 with up to 8 taps the body of the carry kernel (one
+// channel pair per thread, the FIR halo carried in registers, warp-local DFT
+// stages), else the body of the row kernel (first DFT stage on the FIR's
+// registers).  When the wide queue is empty, the CTA splits into two groups of
+// 256 threads, each with half of the shared memory and its own named barrier,
+// and each group pulls narrow tiles from the second counter and runs them
+// independently with the generic body.
 // Both counters are reset by one memset before the launch, so the pair can
 // be captured in a CUDA graph.  The body of each tile is chosen by the beam's
 // (C, tap bucket) class.  Complex int8 input, complex FP32 output: the
@@ -25,8 +26,10 @@
 #include <cstring>
 #include <mutex>
 #include <new>
+#include <queue>
 #include <unordered_map>
 #include <unordered_set>
+#include <utility>
 #include <vector>
 
 #include "../../include/ppf.h"
@@ -74,8 +77,8 @@ struct BeamsArgs {
 
 template <int CI> constexpr int class_threads() { return CI >= kFirstWide ? kBeamThreads : kNarrowThreads; }
 // C = 1024 (the whole CTA): the carry kernel's body, whose
-// one-channel-pair-per-thread shape matches the group; the other classes
-// run fwd_range
+// one-channel-pair-per-thread shape matches the group, in its form without the
+// halo-only pass at the end of each tile; the other classes run fwd_range
 template <int CI, int TI>
 constexpr bool class_carry() {
     constexpr int C = kBeamC[CI], TM = kBeamTM[TI];
@@ -87,10 +90,12 @@ constexpr bool class_carry() {
     }
 }
 
-// C = 2048 and 4096 (the whole CTA): the row kernel's body (24 beams of 1024 to
-// 32768 spectra, 7.4 GB in and out: 5.34 -> 3.94 ms)
+// C = 2048 and 4096, and 1024 with 9 to 16 taps as in ppf_execute (the whole CTA):
+// the row kernel's body (24 beams of 1024 to 32768 spectra, 7.4 GB in and out: 5.34 ->
+// 3.94 ms; 152 beams of 2^20 samples at C = 1024, T = 16: the carry body without the
+// halo-only pass 1298 us, with it 788)
 template <int CI, int TI>
-constexpr bool class_row() { return kBeamC[CI] >= 2048; }
+constexpr bool class_row() { return kBeamC[CI] >= 2048 || (kBeamC[CI] == 1024 && kBeamTM[TI] > 8); }
 
 template <int CI, int TI, class GRP>
 __device__ __forceinline__ bool beam_tile(const BeamsArgs& a, const BeamDesc& d, const BeamTile& t,
@@ -111,7 +116,7 @@ __device__ __forceinline__ bool beam_tile(const BeamsArgs& a, const BeamDesc& d,
     if constexpr (class_row<CI, TI>())
         return row_range<C, TM, IN_CI8, OUT_CF32>(fa, d.in, d.out, t.lo, t.hi, smem);
     else if constexpr (class_carry<CI, TI>())
-        return carry_range<C, TM, IN_CI8, OUT_CF32, false, GRP, true>(fa, d.in, d.out, t.lo, t.hi, smem);
+        return carry_range<C, TM, IN_CI8, OUT_CF32, false, GRP, true, true>(fa, d.in, d.out, t.lo, t.hi, smem);
     else
         return fwd_range<C, TM, IN_CI8, OUT_CF32, class_threads<CI>(), GRP>(fa, d.in, d.out, t.lo, t.hi, smem);
 }
@@ -142,7 +147,7 @@ constexpr int class_smem_max() {
 template <int CI, int TI>
 constexpr int class_batch(int cls) {
     if (cls == CI * kNumTM + TI)
-        return class_row<CI, TI>() ? RowShape<kBeamC[CI >= 5 ? CI : 5], kBeamTM[TI], IN_CI8>::B
+        return class_row<CI, TI>() ? RowShape<kBeamC[CI >= kFirstWide ? CI : kFirstWide], kBeamTM[TI], IN_CI8>::B
              : class_carry<CI, TI>() ? CarryShape<kBeamC[CI], kBeamTM[TI], IN_CI8>::B
                                      : FwdShape<kBeamC[CI], kBeamTM[TI], IN_CI8, class_threads<CI>()>::B;
     if constexpr (TI + 1 < kNumTM) return class_batch<CI, TI + 1>(cls);
@@ -241,40 +246,106 @@ static bool valid_beams(ppf_beams_t b) {
     return g_beams.count(b) != 0 && b->magic == kBeamsMagic;
 }
 
-// Cut every beam into tiles of about tile_samples samples (whole output
-// batches of its class); wide tiles (C >= 2048) first, each queue sorted by
-// work (samples x tap bucket) largest first.
-static ppf_status build_tiles(ppf_beams_t b, long long tile_samples) {
-    std::vector<ppf::BeamTile> tiles[2];
-    std::vector<long long> weight[2];
-    for (int i = 0; i < b->n_beams; ++i) {
-        const ppf::BeamDesc& d = b->host[i];
-        const int q = d.C >= ppf::kBeamC[ppf::kFirstWide] ? 0 : 1;
-        const long long B = ppf::class_batch<0, 0>(d.cls);
-        const long long nbt = (d.n_spectra + B - 1) / B;
-        long long per = tile_samples / (B * d.C);
-        if (per < 1) per = 1;
-        for (long long lo = 0; lo < nbt; lo += per) {
-            const long long hi = std::min(nbt, lo + per);
-            tiles[q].push_back(ppf::BeamTile{lo, hi, i});
-            weight[q].push_back((hi - lo) * B * d.C * (long long)b->tm[i]);
+// The tiles of one queue with the time each is expected to take (us), longest first.
+struct TileQueue {
+    std::vector<ppf::BeamTile> tiles;
+    std::vector<double> us;
+};
+
+// Expected time of `samples` samples on a wide tile's CTA or a narrow tile's half
+// of one, and what a tile takes beside that (tables, barriers, the first copy),
+// fitted to sets of equal beams of every C and T (within 15 %).
+static double tile_us(bool wide, int tm, double samples) {
+    return 3.6 + samples / (1 << 20) * (wide ? 350. + 27. * tm : 740. + 30. * tm);
+}
+
+// Cut every beam into equal tiles of at most about tile_samples samples (whole
+// output batches of its class): q[0] wide tiles (C >= 1024), q[1] narrow ones.
+static void cut_tiles(ppf_beams_t b, long long tile_samples, TileQueue q[2]) {
+    for (int w = 0; w < 2; ++w) {
+        std::vector<std::pair<double, ppf::BeamTile>> all;
+        for (int i = 0; i < b->n_beams; ++i) {
+            const ppf::BeamDesc& d = b->host[i];
+            const bool wide = d.C >= ppf::kBeamC[ppf::kFirstWide];
+            if (wide != (w == 0)) continue;
+            const long long B = ppf::class_batch<0, 0>(d.cls);
+            const long long nbt = (d.n_spectra + B - 1) / B;
+            const long long per = std::max(1ll, tile_samples / (B * d.C));
+            const long long n = (nbt + per - 1) / per, whole = nbt / n, more = nbt % n;   // `more` tiles have one batch more
+            for (long long t = 0, lo = 0; t < n; ++t) {
+                const long long hi = lo + whole + (t < more ? 1 : 0);
+                all.push_back({tile_us(wide, b->tm[i], (double)((hi - lo) * B * d.C)), ppf::BeamTile{lo, hi, i}});
+                lo = hi;
+            }
+        }
+        std::stable_sort(all.begin(), all.end(), [](const auto& x, const auto& y) { return x.first > y.first; });
+        q[w] = TileQueue{};
+        for (const auto& t : all) {
+            q[w].us.push_back(t.first);
+            q[w].tiles.push_back(t.second);
         }
     }
-    std::vector<ppf::BeamTile> sorted;
-    for (int q = 0; q < 2; ++q) {
-        std::vector<size_t> order(tiles[q].size());
-        for (size_t i = 0; i < order.size(); ++i) order[i] = i;
-        std::stable_sort(order.begin(), order.end(), [&](size_t x, size_t y) { return weight[q][x] > weight[q][y]; });
-        for (size_t i : order) sorted.push_back(tiles[q][i]);
+}
+
+// When the last tile ends: the CTAs pull the wide tiles, then their halves the narrow ones.
+static double tiles_end(const TileQueue q[2], int ctas) {
+    using Heap = std::priority_queue<double, std::vector<double>, std::greater<double>>;
+    double end = 0.;
+    auto pull = [&](Heap& free_at, const std::vector<double>& us) {
+        for (double t : us) {
+            const double e = free_at.top() + t;
+            free_at.pop();
+            free_at.push(e);
+            end = std::max(end, e);
+        }
+    };
+    Heap cta, half;
+    for (int i = 0; i < ctas; ++i) cta.push(0.);
+    pull(cta, q[0].us);
+    for (; !cta.empty(); cta.pop()) {
+        half.push(cta.top());
+        half.push(cta.top());
     }
+    pull(half, q[1].us);
+    return end;
+}
+
+// Tile size of a new plan: of 2^20, 2^19 .. 2^13 samples the smallest with which the
+// end is the earliest or within 1 % of it (at C = 4096, T = 16, 152 beams of 2^20
+// samples in one tile each run in step and take 876 us, in two each 774).  Small tiles let few or uneven beams occupy every SM and end together, at a
+// few us each; where beams of one size fill the SMs evenly they only cost (608
+// beams of 2^16 samples at C = 64, T = 4: 122 us whole, 162 in tiles of 2^13).
+// Against a fixed 2^20: 24 beams, 742 M samples 3.80 -> 3.10 ms; 12 beams, 31 M 1.10
+// -> 0.17 ms; 96 beams, 11.5 G unchanged (39 ms).
+static long long pick_tile_samples(ppf_beams_t b) {
+    long long best = 1ll << 20;
+    double best_end = 0.;
+    for (long long ts = 1ll << 20; ts >= 1ll << 13; ts >>= 1) {
+        TileQueue q[2];
+        cut_tiles(b, ts, q);
+        const double end = tiles_end(q, b->sms * b->occupancy);
+        if (best_end == 0. || end < 1.01 * best_end) {
+            best = ts;
+            best_end = best_end == 0. ? end : std::min(end, best_end);
+        }
+        if (q[0].us.size() + q[1].us.size() > 64ull * b->sms) break;   // smaller ones would only add to their cost
+    }
+    return best;
+}
+
+static ppf_status build_tiles(ppf_beams_t b, long long tile_samples) {
+    TileQueue q[2];
+    cut_tiles(b, tile_samples, q);
+    std::vector<ppf::BeamTile> sorted = q[0].tiles;
+    sorted.insert(sorted.end(), q[1].tiles.begin(), q[1].tiles.end());
     if (b->d_tiles) cudaFree(b->d_tiles);
     b->d_tiles = nullptr;
     cudaError_t ce = cudaMalloc(&b->d_tiles, sizeof(ppf::BeamTile) * std::max<size_t>(1, sorted.size()));
     if (ce == cudaSuccess)
         ce = cudaMemcpy(b->d_tiles, sorted.data(), sizeof(ppf::BeamTile) * sorted.size(), cudaMemcpyHostToDevice);
     if (ce != cudaSuccess) return bcuda(ce, "ppf_beams: tiles");
-    b->n_wide = (long long)tiles[0].size();
-    b->n_narrow = (long long)tiles[1].size();
+    b->n_wide = (long long)q[0].tiles.size();
+    b->n_narrow = (long long)q[1].tiles.size();
     b->tile_samples = tile_samples;
     return PPF_OK;
 }
@@ -372,14 +443,7 @@ extern "C" ppf_status ppf_beams_plan(ppf_beams_t* out, int n_beams, const int* C
         b->host[i].taps = b->d_taps + taps_off[i];
         b->host[i].tw = b->d_tw + tw_off[C[i]];
     }
-    // About 24 tiles per CTA, so that the last ones end together and a few beams
-    // occupy every SM; at most 2^20 samples, where a tile's set-up no longer
-    // shows, and at least 2^13 (a batch or two).  Against a fixed 2^20: 24 beams,
-    // 742 M samples 3.80 -> 3.10 ms; 12 beams, 31 M 1.10 -> 0.17 ms; 96 beams,
-    // 11.5 G unchanged (39 ms).
-    long long samples = 0;
-    for (int i = 0; i < n_beams; ++i) samples += n_spectra[i] * C[i];
-    ppf_status s = build_tiles(b, std::min(1ll << 20, std::max(1ll << 13, samples / (24ll * sms))));
+    ppf_status s = build_tiles(b, pick_tile_samples(b));
     if (s != PPF_OK) {
         ppf_beams_destroy(b);
         return s;
