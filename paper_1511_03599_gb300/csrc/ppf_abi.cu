@@ -117,11 +117,15 @@ bool twiddles(int C, std::vector<float>& pairs) {
     }
 }
 
-// Let every kernel of an entry use its dynamic shared memory.
-cudaError_t allow_smem(const ppf::FwdEntry& e) {
+// Let every kernel of an entry use its dynamic shared memory; fills in small_ctas.
+cudaError_t allow_smem(ppf::FwdEntry& e) {
     const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
     cudaError_t ce = cudaFuncSetAttribute(e.fn, attr, e.smem);
-    if (ce == cudaSuccess && e.small_batch > 0) ce = cudaFuncSetAttribute(e.small_fn, attr, e.small_smem);
+    if (ce == cudaSuccess && e.small_batch > 0) {
+        ce = cudaFuncSetAttribute(e.small_fn, attr, e.small_smem);
+        if (ce == cudaSuccess)
+            ce = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&e.small_ctas, e.small_fn, e.threads, e.small_smem);
+    }
     if (ce == cudaSuccess && e.short_fn != nullptr) ce = cudaFuncSetAttribute(e.short_fn, attr, e.smem);
     return ce;
 }
@@ -341,6 +345,26 @@ static long long work_units(long long resident, long long n_streams, long long b
     return std::max<long long>(1, std::min<long long>(resident, total));
 }
 
+// Whether a call runs on the entry's small batches, and on how many CTAs.  It does
+// where each SM gets at most one of them; on the row and long-tap kernels also where
+// the CTA with the most batches ends sooner with them: streams of fewer spectra
+// than a batch, or a last batch that is nearly empty.  A small batch takes 0.2 to
+// 0.45 of the time of a large one (row kernel, up to 16 taps) or 0.3 to 0.6 (beyond,
+// and long-tap kernel).  us, large -> small: C = 1024 T = 4 FP32, 3000 streams of one
+// spectrum 164 -> 75; C = 384 T = 4 int8 143 -> 56; C = 256 T = 24 int8, 3000 of 9 spectra
+// 111 -> 62; C = 128 T = 24, one of 8000 11.0 -> 8.5.
+static bool run_small(const ppf::FwdEntry& e, int resident, int sms, long long n, long long n_streams, long long* grid) {
+    if (e.small_batch <= 0) return false;
+    const long long small = n_streams * ((n + e.small_batch - 1) / e.small_batch);
+    const long long at_once = (long long)sms * e.small_ctas;
+    *grid = std::min(small, std::max<long long>(at_once, sms));
+    if (small <= sms) return true;
+    if (!(e.variant & (64 | 128)) || e.small_ctas < 1) return false;
+    const long long large = n_streams * ((n + e.batch - 1) / e.batch);
+    const double time = (e.variant & 64) || e.tap_bucket > 16 ? 0.6 : 0.45;
+    return time * (double)((small + at_once - 1) / at_once) < (double)((large + resident - 1) / resident);
+}
+
 // Launch one of an entry's kernels: `resident` CTAs of e.fn fit the device at once.
 static ppf_status launch_entry(const ppf::FwdEntry& e, int resident, int sms, const ppf::FwdArgs& a, const char* what,
                                cudaStream_t st) {
@@ -349,11 +373,7 @@ static ppf_status launch_entry(const ppf::FwdEntry& e, int resident, int sms, co
     const int unit = e.cluster > 0 ? e.cluster : 1;                // CTAs per work unit
     auto* launch = e.launch;
     long long grid;
-    // a call that gives each SM at most one small batch runs on those
-    const long long n_small = e.small_batch > 0 && n <= sms * (long long)e.small_batch
-                                  ? n_streams * ((n + e.small_batch - 1) / e.small_batch) : sms + 1ll;
-    if (n_small <= sms) {
-        grid = n_small;
+    if (run_small(e, resident, sms, n, n_streams, &grid)) {
         launch = e.small_launch;
     } else if ((e.variant & 4) && e.cluster == 0) {
         // carry kernel: the same number of CTAs on every stream, one wave if

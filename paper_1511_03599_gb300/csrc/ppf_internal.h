@@ -27,14 +27,15 @@ struct FwdEntry {
     const void* fn;  // kernel function (for occupancy queries and attributes)
     cudaError_t (*launch)(const FwdArgs&, int grid, cudaStream_t);
     int cluster;     // CTAs per thread-block cluster (0: none); grid counts CTAs
-    // the same arithmetic in smaller batches, for calls too short to give every
-    // SM one of the batches above (batch 0: none); same threads per CTA
+    // the same arithmetic in smaller batches, for calls or streams too short for
+    // the batches above (batch 0: none); same threads per CTA
     int small_batch, small_smem;
     const void* small_fn;
     cudaError_t (*small_launch)(const FwdArgs&, int grid, cudaStream_t);
     // carry kernel: the form for at most kCarryShort batches per CTA (nullptr: none)
     const void* short_fn;
     cudaError_t (*short_launch)(const FwdArgs&, int grid, cudaStream_t);
+    int small_ctas;  // resident CTAs of small_fn per SM (set by the plan)
 };
 
 // Resident clusters of a cluster kernel entry (persistent grid): the most
