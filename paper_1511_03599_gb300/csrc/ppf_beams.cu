@@ -36,13 +36,6 @@
 #include "ppf_fwd.cuh"
 #include "ppf_internal.h"
 
-// C = 512 tiles on the carry body of a half-CTA group measured 2 % slower on
-// the C <= 512 beams of the 96-beam set than on fwd_range (and equal on the
-// whole set), so they run fwd_range unless this is set.
-#ifndef PPF_BEAMS_CARRY512
-#define PPF_BEAMS_CARRY512 0
-#endif
-
 namespace ppf {
 
 constexpr int kBeamThreads = 512;                 // one CTA per SM
@@ -78,11 +71,12 @@ struct BeamsArgs {
 template <int CI> constexpr int class_threads() { return CI >= kFirstWide ? kBeamThreads : kNarrowThreads; }
 // C = 1024 (the whole CTA): the carry kernel's body, whose
 // one-channel-pair-per-thread shape matches the group, in its form without the
-// halo-only pass at the end of each tile; the other classes run fwd_range
+// halo-only pass at the end of each tile; the other classes run fwd_range (the
+// carry body on half a CTA measured 2 % slower at C = 512)
 template <int CI, int TI>
 constexpr bool class_carry() {
     constexpr int C = kBeamC[CI], TM = kBeamTM[TI];
-    if constexpr ((C == 512 && PPF_BEAMS_CARRY512) || C == 1024) {
+    if constexpr (C == 1024) {
         using S = CarryShape<C, TM, IN_CI8>;
         return S::OK && S::NT == class_threads<CI>();
     } else {

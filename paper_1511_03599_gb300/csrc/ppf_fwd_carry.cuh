@@ -170,6 +170,7 @@ __device__ __forceinline__ bool carry_range(const FwdArgs& args, const void* in,
     // (341 -> 352); elsewhere it measured -8 .. +1 % (the waits cost registers where
     // those are short, and CTAs that share an SM already fill each other's gaps).
     constexpr bool FREE = S::FREE_RUN && !FIRONLY;
+    static_assert(!FREE || std::is_same<GRP, CtaGroup>::value, "the one-barrier form synchronises the whole CTA");
     constexpr int NBAR = FREE ? 4 : 3;
     uint64_t* bars = reinterpret_cast<uint64_t*>(ring + 2 * S::SLOTB);     // slots 0 and 1, never, ybuf read (FREE)
     volatile int* sflag = reinterpret_cast<volatile int*>(bars + NBAR);
