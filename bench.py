@@ -164,7 +164,9 @@ class ClockSampler:
 
 
 def kernel_name(w, info):
-    name = "pfb_fwd_carry_kernel" if info["variant"] & 4 else "pfb_fwd_row_kernel" if info["variant"] & 128 else "pfb_fwd_kernel"
+    v = info["variant"]            # the cluster kernel carries its halo too: its bit first
+    name = ("pfb_fwd_cluster_kernel" if v & 16 else "pfb_fwd_row_kernel" if v & 128 else
+            "pfb_fwd_longtap_kernel" if v & 64 else "pfb_fwd_carry_kernel" if v & 4 else "pfb_fwd_kernel")
     return f"{name}<{w.C},{info['tap_bucket']},{w.in_dtype},{w.out_dtype}>"
 
 
