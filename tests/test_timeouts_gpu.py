@@ -1,8 +1,8 @@
-"""A bounded device wait that runs out (a barrier that nothing completes, 2 ms) in
-the kernels of the three-pass adjoint: the status is reported, no gradient looks
-complete, and the next call is right.  At C >= 64 the inverse DFT gives up and the
-second pass must not use its rows; at C = 32, whose inverse DFT waits for
-nothing, the second pass gives up itself.
+"""A bounded device wait that runs out (a barrier that nothing completes, 2 ms): the
+status is reported, no result that depends on it looks complete, the launch ends at
+once, and the next call is right.  In the three-pass adjoint at C >= 64 the inverse
+DFT gives up and the second pass must not use its rows; at C = 32, whose inverse DFT
+waits for nothing, the second pass gives up itself.
 """
 import numpy as np
 import pytest
@@ -82,3 +82,32 @@ def test_a_launch_that_gave_up_ends_at_once(ppf, C, T, in_dtype, S, back):
         with pytest.raises(ppf.PPFError):
             plan.check_device()
         assert 1.5 <= ms <= good + 30.0
+
+
+# variant bits: 1 raw rows through a TMA ring, 4 carry kernel, 16 cluster kernel, 64 long-tap
+# kernel, 128 row kernel
+@pytest.mark.parametrize("C,T,in_dtype,S,family,ring", [(32, 8, "ci8", 5000, 0, 1), (32, 16, "cf32", 300, 0, 1),
+                                                        (4096, 8, "ci8", 3000, 128, 1), (3072, 8, "cf32", 3000, 128, 0),
+                                                        (1024, 4, "cf32", 6000, 128, 0), (3072, 8, "cf32", 9, 128, 0),
+                                                        (1024, 8, "ci8", 9000, 4, 1), (512, 8, "ci8", 30, 4, 1),
+                                                        (512, 64, "ci16", 40, 64, 1)])
+def test_forward_reports_a_timeout(ppf, C, T, in_dtype, S, family, ring):
+    """The give-up path of each forward body, named by its kernel family: the generic
+    kernel's ring, the row kernel with its ring, staged and direct, in whole and small
+    batches, the carry kernel's one-barrier and short forms, the long-tap kernel's."""
+    h = synth.design_taps(C, T)
+    x = synth.stream(C, S + T - 1, in_dtype, SIGMA[in_dtype], 9550 + C)
+    xd = torch.from_numpy(x).cuda()
+    with ppf.Plan(C, T, h, in_dtype, "c64") as plan:
+        v = plan.info()["variant"]
+        assert v & (4 | 16 | 64 | 128) == family and v & 1 == ring
+        plan.set_debug_flags(1)
+        plan(xd)
+        with pytest.raises(ppf.PPFError) as ei:
+            plan.check_device()
+        assert ei.value.status == 5
+        plan.set_debug_flags(0)
+        got = plan(xd).cpu().numpy()
+        plan.check_device()
+    idx = np.unique(np.linspace(0, S - 1, 40).astype(np.int64))
+    assert oracle.rel_l2_max_per_spectrum(got[idx], oracle.pfb_spectra(x, h, C, T, idx)) <= 1e-5
