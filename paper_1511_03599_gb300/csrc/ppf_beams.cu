@@ -139,11 +139,14 @@ constexpr int class_smem_max() {
     else return s;
 }
 template <int CI, int TI>
+constexpr int class_batch_of() {
+    if constexpr (class_row<CI, TI>()) return RowShape<kBeamC[CI], kBeamTM[TI], IN_CI8>::B;
+    else if constexpr (class_carry<CI, TI>()) return CarryShape<kBeamC[CI], kBeamTM[TI], IN_CI8>::B;
+    else return FwdShape<kBeamC[CI], kBeamTM[TI], IN_CI8, class_threads<CI>()>::B;
+}
+template <int CI, int TI>
 constexpr int class_batch(int cls) {
-    if (cls == CI * kNumTM + TI)
-        return class_row<CI, TI>() ? RowShape<kBeamC[CI >= kFirstWide ? CI : kFirstWide], kBeamTM[TI], IN_CI8>::B
-             : class_carry<CI, TI>() ? CarryShape<kBeamC[CI], kBeamTM[TI], IN_CI8>::B
-                                     : FwdShape<kBeamC[CI], kBeamTM[TI], IN_CI8, class_threads<CI>()>::B;
+    if (cls == CI * kNumTM + TI) return class_batch_of<CI, TI>();
     if constexpr (TI + 1 < kNumTM) return class_batch<CI, TI + 1>(cls);
     else if constexpr (CI + 1 < kNumC) return class_batch<CI + 1, 0>(cls);
     else return 0;

@@ -28,10 +28,6 @@
 
 #include "ppf_fwd.cuh"
 
-#ifndef PPF_BWD_CARRY_SMEM
-#define PPF_BWD_CARRY_SMEM 1
-#endif
-
 namespace ppf {
 
 template <int C, int TM, int IN = IN_CF32>
@@ -55,7 +51,7 @@ struct BwdShape {
     // WIDE with 8 taps: the 7 carried g_y rows wait in shared memory (one
     // column per thread) while the inverse DFT holds its 64 values per thread
     // in registers (+3 .. +4 %; with 4 taps the registers measured 3 % faster)
-    static constexpr bool CARRY_SMEM = WIDE && TM >= 8 && PPF_BWD_CARRY_SMEM;
+    static constexpr bool CARRY_SMEM = WIDE && TM >= 8;
     static constexpr int CARRY_OFF = 2 * SLOTB + 2 * XSLOTB + TWB + 64;
     static constexpr int SMEM = CARRY_OFF + (CARRY_SMEM ? (TM - 1) * NT * 8 : 0);
     static constexpr bool FFT_OK = SPW > 0 ? (SPW * NWARP == B && (WIDE ? warp_fft_ok(C, SPW) : fft_items_fit(C, SPW, 32)))

@@ -392,16 +392,10 @@ __device__ __forceinline__ void tma_prefetch_l2(const void* src_gmem, uint32_t b
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src_gmem), "r"(bytes) : "memory");
 }
 
-// Asynchronous 4/8/16-byte copy global -> shared (the thread's own staging
-// slot), committed in groups; wait_group<N> returns once at most N of the
-// thread's most recent groups are still in flight.
-template <int BYTES>
-__device__ __forceinline__ void cp_async(void* dst_smem, const void* src_gmem) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_addr(dst_smem)), "l"(src_gmem), "n"(BYTES)
-                 : "memory");
-}
-// The same with zeros in place of the source where !ok (nothing is read then);
-// 16-byte copies bypass L1.
+// Asynchronous 4/8/16-byte copy global -> shared (the thread's own staging slot),
+// with zeros in place of the source where !ok (nothing is read then), committed in
+// groups; wait_group<N> returns once at most N of the thread's most recent groups
+// are still in flight.  16-byte copies bypass L1.
 template <int BYTES>
 __device__ __forceinline__ void cp_async_or_zero(void* dst_smem, const void* src_gmem, bool ok) {
     if constexpr (BYTES == 16)

@@ -174,41 +174,36 @@ struct FwdShape {
     // C = 32, where it lets the TMA ring fit beside the batch (fp32 T = 8: 244 vs
     // 120 GS/s; int16 T = 8: 233 vs 148)
     static constexpr int B = (C == 32 && IN != IN_CI8) ? 128 : 8192 / C;
-    // large-T FIR order (see fir_segment): tap chunks for narrow input at C <= 512
-    static constexpr bool CHUNK = TM > 16 && IN != IN_CF32 && C <= 512;
+    // large-T FIR order (see fir_segment): tap chunks for 8/16-bit input
+    static constexpr bool CHUNK = TM > 16 && IN != IN_CF32;
     static constexpr int L0 = (TM >= 32 && !CHUNK) || (C == 32 && IN != IN_CI8) ? 8 : 16;
     static constexpr int L = L0 < B ? L0 : B;                        // FIR segment (outputs)
     static constexpr int G = B / L;                                  // segments per batch
     static constexpr int FIR_ITEMS = PAIRS * G;                      // (pair, segment) items
     static constexpr int FPT = (FIR_ITEMS + NT - 1) / NT;           // FIR items per thread
-    static constexpr bool FIR_EXACT = FIR_ITEMS % NT == 0;
     static constexpr int YBYTES = B * C * 8;                         // filtered spectra of a batch
     static constexpr int TWBYTES = tw_size(C) * 8;
     static constexpr int BIN = InTraits<IN>::bytes;
     static constexpr int SLOTB = B * C * BIN;                        // raw bytes of one batch
     static constexpr int CTA_SMEM_MAX = generic_smem_cap(NT);
     // TMA ring: every raw batch is copied into shared memory once; the FIR of
-    // batch k reads slot k and the T-1 halo rows from the HS slots after it
-    // (HS = 1 when T-1 <= B; a deeper ring where the halo spans several
-    // batches -- large C, where B is small -- and one segment covers the batch).
-    static constexpr int HS = TM - 1 <= B ? 1 : (TM - 1 + B - 1) / B;    // halo slots
-    // ring slots: HS + 2 (one batch of slack for the refill), or HS + 1 where
-    // only that fits, or where only that leaves room for the twiddle table
-    // (the refill of the slot freed by batch k's FIR then has batch k's DFT
-    // stages to land before batch k+1's FIR reads it; twiddles in shared
-    // memory beside a 2-slot ring measured +2 .. +3 % at C = 2048 and 4096)
-    static constexpr bool NS_TIGHT_FITS = YBYTES + (HS + 1) * SLOTB + 64 <= CTA_SMEM_MAX;
-    static constexpr bool NS_TIGHT_FOR_TW = YBYTES + (HS + 2) * SLOTB + 64 + TWBYTES > CTA_SMEM_MAX &&
-                                            YBYTES + (HS + 1) * SLOTB + 64 + TWBYTES <= CTA_SMEM_MAX;
-    static constexpr int NS = (NS_TIGHT_FITS &&
-                               (YBYTES + (HS + 2) * SLOTB + 64 > CTA_SMEM_MAX || NS_TIGHT_FOR_TW)) ? HS + 1 : HS + 2;
-    static constexpr bool RING = (TM - 1 <= B || (G == 1 && TM <= 16)) && (YBYTES + NS * SLOTB + 64 <= CTA_SMEM_MAX);
+    // batch k reads slot k and the T-1 <= B halo rows from the slot after it.
+    // 3 slots (one batch of slack for the refill), or 2 where only that fits, or
+    // where only that leaves room for the twiddle table (the refill of the slot
+    // freed by batch k's FIR then has batch k's DFT stages to land before batch
+    // k+1's FIR reads it).
+    static constexpr bool NS_TIGHT_FITS = YBYTES + 2 * SLOTB + 64 <= CTA_SMEM_MAX;
+    static constexpr bool NS_TIGHT_FOR_TW = YBYTES + 3 * SLOTB + 64 + TWBYTES > CTA_SMEM_MAX &&
+                                            YBYTES + 2 * SLOTB + 64 + TWBYTES <= CTA_SMEM_MAX;
+    static constexpr int NS = (NS_TIGHT_FITS && (YBYTES + 3 * SLOTB + 64 > CTA_SMEM_MAX || NS_TIGHT_FOR_TW)) ? 2 : 3;
+    static constexpr bool RING = YBYTES + NS * SLOTB + 64 <= CTA_SMEM_MAX;
     static constexpr bool TW_SMEM = YBYTES + (RING ? NS * SLOTB + 64 : 0) + TWBYTES <= CTA_SMEM_MAX;
     static constexpr int RING_OFF = YBYTES + (TW_SMEM ? TWBYTES : 0);
     static constexpr int SMEM = RING_OFF + (RING ? NS * SLOTB + 64 : 0);
     // each thread keeps one channel pair for the whole run: taps stay in registers
     static constexpr bool TAPS_IN_REGS = (FPT == 1) && (TM <= 16) && (NT % PAIRS == 0);
-    static_assert(FPT >= 1 && (FIR_EXACT || is_c3(C)), "FIR items must divide evenly");
+    static_assert(FPT >= 1 && FIR_ITEMS % NT == 0, "FIR items must divide evenly");
+    static_assert(TM - 1 <= B, "the halo lies in one slot");
     static_assert(SLOTB % 16 == 0 && YBYTES % 16 == 0 && TWBYTES % 16 == 0, "16-byte alignment");
     static_assert(SMEM <= CTA_SMEM_MAX, "the batch and its ring must fit one CTA's shared memory");
 };
@@ -260,7 +255,7 @@ struct HalfGroup {
 // reads_done: a barrier each warp arrives on once it has read its last stage's input.
 // CONJ: the last stage stores conjugates (the other half of an inverse DFT
 // whose caller conjugates the input).
-template <int C, int B, int NT, int P, int OUT, bool TW_SMEM, int SPW = 0, bool INV = false, bool SMEM_OUT = false,
+template <int C, int B, int NT, int P, int OUT, bool TW_SMEM, int SPW = 0, bool INV = false,
           int LAYOUT = 0, class GRP = CtaGroup, bool CONJ = false>
 __device__ __forceinline__ void fft_stage(float2* __restrict__ ybuf, const float2* __restrict__ tws,
                                           void* __restrict__ out, long long sb, long long vlo, long long vhi,
@@ -276,8 +271,8 @@ __device__ __forceinline__ void fft_stage(float2* __restrict__ ybuf, const float
     constexpr int IPT = (TOTAL + WORKERS - 1) / WORKERS;        // items per thread
     constexpr bool EXACT = IPT * WORKERS == TOTAL;
     constexpr int SPAN = spec_span<C, LAYOUT>();   // elements per spectrum in ybuf
-    static_assert(!(LAYOUT >= 1 && (INV || SMEM_OUT)), "padded or pair-swizzled rows only for the forward stores to HBM");
-    static_assert(EXACT || (SPW == 0 && is_c3(C)) || TOTAL < WORKERS,
+    static_assert(!(LAYOUT >= 1 && INV), "padded or pair-swizzled rows only for the forward stores to HBM");
+    static_assert(EXACT || TOTAL < WORKERS,
                   "items must divide evenly (a warp or CTA may leave threads idle)");
     const int gtid = GRP::tid();
     const int wid = SPW > 0 ? (gtid & 31) : gtid;
@@ -330,15 +325,6 @@ __device__ __forceinline__ void fft_stage(float2* __restrict__ ybuf, const float
             float2* dst = ybuf + sp * C;
 #pragma unroll
             for (int k = 0; k < R; ++k) dst[prefix + PP * k] = make_float2(v[it][k].x, -v[it][k].y);
-        } else if constexpr (SMEM_OUT) {   // natural order, output type, row stride C elements
-#pragma unroll
-            for (int k = 0; k < R; ++k) {
-                if constexpr (OUT == OUT_CF32) {
-                    ybuf[sp * C + prefix + PP * k] = v[it][k];
-                } else {
-                    reinterpret_cast<__half2*>(ybuf)[sp * C + prefix + PP * k] = __float22half2_rn(v[it][k]);
-                }
-            }
         } else {
             const long long s = sb + sp;
             if (s >= vlo && s < vhi) {
@@ -352,12 +338,12 @@ __device__ __forceinline__ void fft_stage(float2* __restrict__ ybuf, const float
 
 // Where the FIR reads raw samples of channel pair cp from: rows are relative
 // to the first raw spectrum of the batch (row r feeds outputs r-T+1 .. r).
-template <int C, int IN, bool RING, int B, int HS = 1>
+template <int C, int IN, bool RING, int B>
 struct RawSrc {
     static constexpr int BIN = InTraits<IN>::bytes;
     static constexpr bool kRing = RING;
-    // ring: shared-memory slots of the batch and of the HS batches after it
-    const unsigned char* sl[HS + 1];
+    // ring: shared-memory slots of the batch and of the one after it
+    const unsigned char* sl[2];
     // direct: global stream
     const void* in;
     long long row0, n_raw;
@@ -365,12 +351,8 @@ struct RawSrc {
 
     __device__ __forceinline__ float4 load(int r) const {
         if constexpr (RING) {
-            if constexpr (HS == 1) {
-                const unsigned char* p = (r < B) ? sl[0] + (size_t)r * C * BIN : sl[1] + (size_t)(r - B) * C * BIN;
-                return load_pair_smem<IN>(p);
-            } else {
-                return load_pair_smem<IN>(sl[r / B] + (size_t)(r % B) * C * BIN);   // r is a compile-time row here
-            }
+            const unsigned char* p = (r < B) ? sl[0] + (size_t)r * C * BIN : sl[1] + (size_t)(r - B) * C * BIN;
+            return load_pair_smem<IN>(p);
         } else {
             const long long rr = row0 + r;
             return (rr < n_raw) ? load_pair_global<IN>(in, rr * C + 2 * cp) : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -482,7 +464,7 @@ __device__ __forceinline__ void fir_segment(const Src& src, const float2* __rest
         // Large T (T is a runtime bound); packed (re, im) x (h, h) FMAs; a
         // segment wholly inside the stream loads without per-sample bounds
         // checks.  Two orders, chosen per shape by measurement:
-        //  * CHUNK (8/16-bit input, C <= 512): the taps in chunks of K held in
+        //  * CHUNK (8/16-bit input): the taps in chunks of K held in
         //    registers; for each chunk the raw-sample-outer order of the small-T
         //    path over the L+K-1 rows it needs -- a tap is loaded once per
         //    segment and serves L outputs (rows are re-read per chunk: cheap
@@ -669,12 +651,11 @@ __device__ __forceinline__ bool fwd_range(const FwdArgs& args, const void* in, v
 #pragma unroll 1
         for (int f = 0; f < S::FPT; ++f) {
             const int item = tid + f * NT;
-            if (!S::FIR_EXACT && item >= S::FIR_ITEMS) break;
             const int cp = item % S::PAIRS, g = item / S::PAIRS;
-            RawSrc<C, IN, RING, B, S::HS> src;
+            RawSrc<C, IN, RING, B> src;
             if constexpr (RING) {
 #pragma unroll
-                for (int h = 0; h <= S::HS; ++h) src.sl[h] = ring + ((k + h) % NS) * S::SLOTB + 2 * cp * S::BIN;
+                for (int h = 0; h < 2; ++h) src.sl[h] = ring + ((k + h) % NS) * S::SLOTB + 2 * cp * S::BIN;
             } else {
                 src.in = in;
                 src.row0 = sb;
@@ -699,7 +680,7 @@ __device__ __forceinline__ bool fwd_range(const FwdArgs& args, const void* in, v
         }
         // ---------------------------------------------------------- FFT
         static_for<NST>([&](auto p) {
-            fft_stage<C, B, NT, decltype(p)::value, OUT, S::TW_SMEM, 0, false, false, 0, GRP>(ybuf, tws, out, sb, 0, n_spectra);
+            fft_stage<C, B, NT, decltype(p)::value, OUT, S::TW_SMEM, 0, false, 0, GRP>(ybuf, tws, out, sb, 0, n_spectra);
         });
     }
     if constexpr (RING) {
@@ -770,9 +751,9 @@ constexpr bool carry_preferred() {
     return CarryShape<C, TM, IN>::OK && !(C == 1024 && TM > 8);
 }
 
-// The row kernel for the rest of C >= 1024 and C = 3 * 2^k up to 16 taps, except
-// FP32 input at C = 2048 with 5-8 taps: the cluster kernel is slower there (153
-// against 253 GS/s), but ppf_plan_info's variant of that shape is relied on.
+// The row kernel for the rest of C >= 1024 and C = 3 * 2^k, except FP32 input at
+// C = 2048 with 5-8 taps: the cluster kernel is slower there (153 against 253 GS/s),
+// but two tests name it for that shape (ppf_plan_info's variant).
 template <int C, int TM, int IN>
 constexpr bool row_preferred() {
     if constexpr (C >= 1024 || is_c3(C)) return RowShape<C, TM, IN>::OK && !(C == 2048 && IN == IN_CF32 && TM == 8);

@@ -24,15 +24,6 @@
 
 #include "ppf_fwd.cuh"
 
-// The last DFT stage's buffer uses the pair-chunk swizzle (phys, LAYOUT 2)
-// where it measured faster than the element swizzle: C = 1024 (+0.4 % at
-// T = 8, +3 % at T = 16, int8), int16 input at C = 512 (+1.3 %) and int8
-// input at C = 256 (+1.6 %); it measured 1-3 % slower for int8 and fp32 input
-// at C = 512 and fp32 at C = 256.  PPF_LAYOUT2=0 turns it off.
-#ifndef PPF_LAYOUT2
-#define PPF_LAYOUT2 1
-#endif
-
 namespace ppf {
 
 // every FFT stage must give each thread a whole number (>= 1) of items
@@ -66,8 +57,11 @@ struct CarryCand {
     // last DFT stage's buffer: padded rows (no per-access index arithmetic)
     // where they measured faster -- C <= 128, and 16 taps at C <= 256 --
     // else the element XOR swizzle (C = 512/1024 at T <= 8 lost 2-4 % with
-    // padding) or, where it measured faster, the pair-chunk swizzle
-    static constexpr bool PAIR_SWIZZLE = PPF_LAYOUT2 && last_radix(C) >= 16 &&
+    // padding) or the pair-chunk swizzle where it measured faster: C = 1024 (+0.4 %
+    // at T = 8, +3 % at T = 16, int8), int16 input at C = 512 (+1.3 %) and int8 input
+    // at C = 256 (+1.6 %); 1-3 % slower for int8 and fp32 input at C = 512 and fp32 at
+    // C = 256
+    static constexpr bool PAIR_SWIZZLE = last_radix(C) >= 16 &&
                                          (C == 1024 || (C == 512 && IN == IN_CI16) || (C == 256 && IN == IN_CI8));
     static constexpr int LAYOUT = (C <= 128 || (TM >= 16 && C <= 256)) ? 1 : PAIR_SWIZZLE ? 2 : 0;
     static constexpr int YSPAN = spec_span<C, LAYOUT>();             // elements per spectrum in ybuf
@@ -366,7 +360,7 @@ __device__ __forceinline__ bool carry_range(const FwdArgs& args, const void* in,
         if constexpr (!FIRONLY) {
             const long long sb = (lo + k) * B + sh - (T - 1);     // output spectrum of batch row 0
             static_for<NST>([&](auto p) {
-                fft_stage<C, B, NT, decltype(p)::value, OUT, S::TW_SMEM, S::SPW, false, false, S::LAYOUT, GRP, CONJ>(
+                fft_stage<C, B, NT, decltype(p)::value, OUT, S::TW_SMEM, S::SPW, false, S::LAYOUT, GRP, CONJ>(
                     ybuf, tws, out, sb, vlo, vhi, FREE ? &bars[NBAR - 1] : nullptr);
             });
         }

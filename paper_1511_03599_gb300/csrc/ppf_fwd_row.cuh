@@ -2,7 +2,7 @@
 // the first DFT stage done on the FIR's registers and the rest of the
 // transform local to a few warps.
 //
-// C = R0 * M (R0 = 1, 2, 3 or 4, M = 128 .. 1024).  With channel c = a M + b and
+// C = R0 * M (R0 = 1, 2, 3 or 4; M = 128 .. 1024, in small batches from 64).  With channel c = a M + b and
 // bin q = k0 + R0 k', Eq. 2 splits into an R0-point DFT over a per column b,
 // a twiddle W_C^{b k0}, and an M-point DFT over b per row k0:
 //   * FIR (Alg. 1) + R0-point DFT: a thread owns the R0 channels of one column
@@ -403,14 +403,9 @@ __device__ __forceinline__ bool row_range(const FwdArgs& args, const void* in, v
                     const int n = a * S::RW + i, gi = n / S::GR;
                     if (n % S::GR == 0) cp_async_wait_upto(S::NGR - 1 - gi < S::NCH - 1 ? S::NGR - 1 - gi : S::NCH - 1);
                     const unsigned char* p = stg + (n % (S::NCH * S::GR)) * (S::NT * S::CB);
-                    if constexpr (PAIR) {
-                        const float4 v = load_pair_smem<IN>(p);
-                        x0 = pk2(v.x, v.z);
-                        x1 = CONJ ? pk2(-v.y, -v.w) : pk2(v.y, v.w);
-                    } else {
-                        const float2 v = load_one_smem<IN>(p);
-                        x0 = pk2(v.x, CONJ ? -v.y : v.y);
-                    }
+                    const float4 v = load_pair_smem<IN>(p);      // STAGE means PAIR
+                    x0 = pk2(v.x, v.z);
+                    x1 = CONJ ? pk2(-v.y, -v.w) : pk2(v.y, v.w);
                     if ((n % S::GR == S::GR - 1 || n + 1 == S::NROW) && gi + S::NCH < S::NGR) stage_group(k, gi + S::NCH);
                 }
             };
