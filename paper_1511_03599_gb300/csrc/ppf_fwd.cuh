@@ -133,10 +133,11 @@ constexpr int tw_offset(int C, int p) {
 }
 constexpr int tw_size(int C) { return tw_offset(C, fft_stages(C) - 1); }
 // The row kernel's tables: W_C^{b k0} at [(k0-1)*M + b], k0 = 1 .. R0-1, then
-// W_M^{b k} of the row's first stage (RA x RB) at [(k-1)*RB + b].  At C = 2048
-// and 4096 they follow the stage tables; elsewhere they are the stage tables.
+// W_M^{b k} of the row's first stage (RA x RB) at [(k-1)*RB + b].  At C = 2048 they
+// follow the stage tables (the cluster kernel's), at C = 4096 they stand alone;
+// elsewhere they are the stage tables.
 constexpr bool row_tw_own(int C) { return C == 2048 || C == 4096; }
-constexpr int row_tw_offset(int C) { return row_tw_own(C) ? tw_size(C) : 0; }
+constexpr int row_tw_offset(int C) { return C == 2048 ? tw_size(C) : 0; }
 constexpr int row_tw_size(int C) {
     return row_tw_own(C) ? (row_r0(C) - 1) * (C / row_r0(C)) + (row_radix(C, 0) - 1) * row_radix(C, 1) : 0;
 }
@@ -857,7 +858,7 @@ inline cudaError_t fir_launch(const FwdArgs& a, int grid, cudaStream_t st) {
 // W_{N_p}^{b k} = exp(-2 pi i b k / N_p), k = 1 .. R_p-1, at
 // [tw_offset(p) + (k-1)*N_{p+1} + b].
 // Entries of the plan's twiddle table for C.
-constexpr int tw_total_float2s(int C) { return tw_size(C) + row_tw_size(C); }
+constexpr int tw_total_float2s(int C) { return (C == 4096 ? 0 : tw_size(C)) + row_tw_size(C); }
 
 // All of them are powers of W_C; each of its C powers is evaluated once.
 template <int C>
@@ -868,7 +869,7 @@ inline void fill_twiddles(float2* host) {
         const long i = e % n * (C / n);
         return make_float2(c[i], -c[(i + C - C / 4) % C]);
     };
-    for (int p = 0; p + 1 < fft_stages(C); ++p) {
+    for (int p = 0; p + 1 < fft_stages(C) && C != 4096; ++p) {
         const int NP = fft_n(C, p), R = fft_radix(C, p), NN = NP / R;
         for (int k = 1; k < R; ++k)
             for (int b = 0; b < NN; ++b) host[tw_offset(C, p) + (k - 1) * NN + b] = power((long)b * k, NP);
