@@ -102,10 +102,12 @@ struct AdjArgs {
     int flags;               // FwdFlags (testing aid)
 };
 
-// ENDS: the steps of the tile at raw row r0 are taps t1, t1 - 1, .., n of them, whose
-// window r0 - t .. r0 - t + kAdjL-1 meets rows 0 .. S-1 of the stream (at least one does).
+// The steps of a tile: taps t1, t1 - 1, .., n of them.  All T, or (ENDS) the ones whose
+// window r0 - t .. r0 - t + kAdjL-1, for the tile at raw row r0, meets rows 0 .. S-1 of
+// the stream (at least one does).
 struct AdjSteps {
     int t1, n;
+    __device__ __forceinline__ explicit AdjSteps(int T) : t1(T - 1), n(T) {}
     __device__ __forceinline__ AdjSteps(long long r0, long long S, int T) {
         t1 = r0 + kAdjL < T ? (int)r0 + kAdjL - 1 : T - 1;
         n = t1 + 1 - (r0 >= S ? (int)(r0 - S) + 1 : 0);
@@ -145,11 +147,12 @@ pfb_bwd_grad_kernel(AdjArgs a, const __grid_constant__ CUtensorMap g_map, const 
 
     grid_dependency_wait();                                               // launched by launch_early
     const int tid = threadIdx.x, lane = tid & 31;
+    const int status = tid == 0 ? *static_cast<volatile int*>(a.err) : 0; // requested here, needed below
     const int c0 = blockIdx.y * NCT;
     const int T = a.T;
     const long long n_raw = a.n_spectra + T - 1;
     const long long tiles = (n_raw + L - 1) / L;
-    int nch = L / RC + (T + RC - 1) / RC;
+    const int nch = L / RC + (T + RC - 1) / RC;
     if (tid == 0) {
         for (int i = 0; i < NS; ++i) {
             mbar_init(&full[i], 1);
@@ -163,7 +166,7 @@ pfb_bwd_grad_kernel(AdjArgs a, const __grid_constant__ CUtensorMap g_map, const 
         for (int t = 0; t < T; ++t) ghs[t * NCT + tid] = 0.f;
     // the status word is set: the inverse DFT (or an earlier launch) gave up, g_y
     // may not have been written
-    const bool failed = __syncthreads_or(tid == 0 && *static_cast<volatile int*>(a.err) != 0);
+    const bool failed = __syncthreads_or(status != 0);
 
     BatchShare share(tiles, a.n_streams, blockIdx.x, gridDim.x);
     long long strm, lo, hi;
@@ -193,13 +196,8 @@ pfb_bwd_grad_kernel(AdjArgs a, const __grid_constant__ CUtensorMap g_map, const 
         bool ok = true;
         while (ok && share.next(strm, lo, hi)) {
             for (long long k = lo; ok && k < hi; ++k) {
-                int t1 = T - 1;
-                if constexpr (ENDS) {
-                    const AdjSteps st(k * L, a.n_spectra, T);
-                    t1 = st.t1;
-                    nch = L / RC + (st.n + RC - 1) / RC;
-                }
-                for (int c = 0; c < nch; ++c) {
+                const AdjSteps st = ENDS ? AdjSteps(k * L, a.n_spectra, T) : AdjSteps(T);
+                for (int c = 0; c < (ENDS ? L / RC + (st.n + RC - 1) / RC : nch); ++c) {
                     if (issued >= NS) ok = mbar_wait_bounded_or(&empty[slot], phase ^ 1, kWaitLimitNs, sdead);
                     ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
@@ -209,8 +207,8 @@ pfb_bwd_grad_kernel(AdjArgs a, const __grid_constant__ CUtensorMap g_map, const 
                         const int u = (c - L / RC) * RC;             // the chunk's first step
                         const bool first = u < 0;
                         mbar_expect_tx(&full[slot], S::GB + (first ? (GH ? RC * NCT * BIN : 0) : RC * NCT * 4));
-                        tma_load_box3(dst, &g_map, c0, (int)(k * L) - t1 + c * RC, (int)strm, &full[slot]);
-                        if (!first) tma_load_box2(dst + S::GB, &tap_map, c0, t1 + 1 - RC - u, &full[slot]);
+                        tma_load_box3(dst, &g_map, c0, (int)(k * L) - (ENDS ? st.t1 : T - 1) + c * RC, (int)strm, &full[slot]);
+                        if (!first) tma_load_box2(dst + S::GB, &tap_map, c0, ENDS ? st.t1 + 1 - RC - u : T - RC - u, &full[slot]);
                         else if (GH) tma_load_box3(dst + S::GB, &x_map, c0, (int)(k * L) + c * RC, (int)strm, &full[slot]);
                     }
                     __syncwarp();
@@ -276,28 +274,23 @@ pfb_bwd_grad_kernel(AdjArgs a, const __grid_constant__ CUtensorMap g_map, const 
                 }
                 release();
             }
-            int t1 = T - 1, n = T;
-            if constexpr (ENDS) {
-                const AdjSteps st(r0, a.n_spectra, T);
-                t1 = st.t1;
-                n = st.n;
-            }
+            const AdjSteps st = ENDS ? AdjSteps(r0, a.n_spectra, T) : AdjSteps(T);
             auto steps = [&](auto edge_tag) {
                 // EDGE (FP32 input): some rows lie outside the stream, and an inf or NaN
                 // sample must not meet their zeros
                 [[maybe_unused]] constexpr bool EDGE = decltype(edge_tag)::value != 0;
 #pragma unroll 1
-                for (int tb = 0; tb < n; tb += L) {
+                for (int tb = 0; tb < (ENDS ? st.n : T); tb += L) {
 #pragma unroll
                     for (int blk = 0; blk < L / RC; ++blk) {
                         const int u0 = tb + blk * RC;
-                        if (u0 >= n) break;
+                        if (u0 >= (ENDS ? st.n : T)) break;
                         wait_full();
 #pragma unroll
                         for (int i = 0; i < RC; ++i) {
                             const int w = blk * RC + i;              // window slot of the oldest row
-                            const int t = t1 - u0 - i;
-                            if (ENDS ? u0 + i >= n : t < 0) break;
+                            const int t = ENDS ? st.t1 - u0 - i : T - 1 - u0 - i;
+                            if (ENDS ? u0 + i >= st.n : t < 0) break;
                             if constexpr (GX) {
                                 const float hv = *reinterpret_cast<const float*>(smem + slot * S::CHUNKB + S::GB +
                                                                                  ((RC - 1 - i) * NCT + tid) * 4);
