@@ -117,15 +117,11 @@ bool twiddles(int C, std::vector<float>& pairs) {
     }
 }
 
-// Let every kernel of an entry use its dynamic shared memory; fills in small_ctas.
-cudaError_t allow_smem(ppf::FwdEntry& e) {
+// Let every kernel of an entry use its dynamic shared memory.
+cudaError_t allow_smem(const ppf::FwdEntry& e) {
     const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
     cudaError_t ce = cudaFuncSetAttribute(e.fn, attr, e.smem);
-    if (ce == cudaSuccess && e.small_batch > 0) {
-        ce = cudaFuncSetAttribute(e.small_fn, attr, e.small_smem);
-        if (ce == cudaSuccess)
-            ce = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&e.small_ctas, e.small_fn, e.threads, e.small_smem);
-    }
+    if (ce == cudaSuccess && e.small_batch > 0) ce = cudaFuncSetAttribute(e.small_fn, attr, e.small_smem);
     if (ce == cudaSuccess && e.short_fn != nullptr) ce = cudaFuncSetAttribute(e.short_fn, attr, e.smem);
     return ce;
 }
@@ -357,9 +353,9 @@ static bool run_small(const ppf::FwdEntry& e, int resident, int sms, long long n
     if (e.small_batch <= 0) return false;
     const long long small = n_streams * ((n + e.small_batch - 1) / e.small_batch);
     const long long at_once = (long long)sms * e.small_ctas;
-    *grid = std::min(small, std::max<long long>(at_once, sms));
+    *grid = std::min(small, at_once);
     if (small <= sms) return true;
-    if (!(e.variant & (64 | 128)) || e.small_ctas < 1) return false;
+    if (!(e.variant & (64 | 128))) return false;
     const long long large = n_streams * ((n + e.batch - 1) / e.batch);
     const double time = (e.variant & 64) || e.tap_bucket > 16 ? 0.6 : 0.45;
     return time * (double)((small + at_once - 1) / at_once) < (double)((large + resident - 1) / resident);

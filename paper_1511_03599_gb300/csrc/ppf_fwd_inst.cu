@@ -26,6 +26,7 @@ static bool make_entry(FwdEntry* e) {
         e->small_smem = S::SMEM;
         e->small_fn = reinterpret_cast<const void*>(&pfb_fwd_row_kernel<PPF_C, TM, IN, OUT, 4>);
         e->small_launch = &row_small_launch<PPF_C, TM, IN, OUT>;
+        e->small_ctas = 1;
     }
     if constexpr (TM == 64) {
         if constexpr (LongShape<PPF_C, IN>::OK) {
@@ -34,6 +35,7 @@ static bool make_entry(FwdEntry* e) {
             e->small_smem = S::SMEM;
             e->small_fn = reinterpret_cast<const void*>(&pfb_fwd_longtap_kernel<PPF_C, IN, OUT, 2>);
             e->small_launch = &longtap_launch<PPF_C, IN, OUT, 2>;
+            e->small_ctas = S::MINB;
         }
     }
     if constexpr (carry_preferred<PPF_C, TM, IN>()) {
@@ -158,6 +160,7 @@ static bool make_idft(FwdEntry* e) {
         e->small_smem = M::SMEM;
         e->small_fn = reinterpret_cast<const void*>(km);
         e->small_launch = &launch_kernel_early<km, M::NT, M::SMEM>;
+        e->small_ctas = 1;
         return true;
     }
 }

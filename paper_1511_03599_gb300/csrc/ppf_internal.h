@@ -35,7 +35,7 @@ struct FwdEntry {
     // carry kernel: the form for at most kCarryShort batches per CTA (nullptr: none)
     const void* short_fn;
     cudaError_t (*short_launch)(const FwdArgs&, int grid, cudaStream_t);
-    int small_ctas;  // resident CTAs of small_fn per SM (set by the plan)
+    int small_ctas;  // resident CTAs of small_fn per SM (at least)
 };
 
 // Resident clusters of a cluster kernel entry (persistent grid): the most
