@@ -238,7 +238,7 @@ def measure_case(w, steps: int, warmup: int, dev, peak: float, fp32_peak: float)
 def measure_fwd_bwd(steps: int, warmup: int, dev):
     """Forward vs forward+backward on the differentiable workload: C=256, T=16,
     64 streams x 8192 spectra of complex64 noise; backward = grad wrt input and
-    taps (inverse DFT, transposed FIR, tap correlation + reduction)."""
+    taps (inverse DFT, transposed FIR and tap correlation, reduction)."""
     import torch
     from paper_1511_03599_gb300 import ppf, synth
     C, T, S, ns = 256, 16, 8192, 64
@@ -318,7 +318,7 @@ def measure_fwd_bwd_headline(plan, w, x, y, steps: int, warmup: int, dev):
 def measure_fwd_bwd_shape(C: int, T: int, in_dtype: str, S: int, steps: int, warmup: int, dev):
     """Forward vs forward + adjoint (both gradients) for one single-stream
     shape; outside the fused adjoint kernel's shapes the adjoint is the
-    three-pass path (inverse DFT, transposed FIR, tap correlation)."""
+    three-pass path (inverse DFT, both gradients, reduction)."""
     import torch
     from paper_1511_03599_gb300 import ppf, synth
     st = torch.cuda.current_stream()
@@ -337,7 +337,7 @@ def measure_fwd_bwd_shape(C: int, T: int, in_dtype: str, S: int, steps: int, war
     del x, G, y
     return {"workload": f"pfb_c{C}_t{T}_s{S}_{in_dtype}_c64", "fwd_ms": t_f, "fwd_bwd_ms": t_fb,
             "fwd_bwd_over_fwd": t_fb / t_f, "bwd_ms": t_fb - t_f, "fwd_launch": fused,
-            "backward": "three-pass: inverse DFT, transposed FIR, tap correlation + fixed-order reduction"}
+            "backward": "three-pass: inverse DFT, both gradients from one pass, fixed-order reduction"}
 
 
 def measure_ablation(plan, x, y, steps: int, warmup: int, dev):
@@ -372,7 +372,7 @@ def measure_ablation(plan, x, y, steps: int, warmup: int, dev):
 def measure_beams(steps: int, dev, seed: int = 4):
     """The multi-beam workload: 96 beams, C in {64..4096}, T in {4, 8, 16},
     spectra per beam uniform in [2^12, 2^17], complex int8 sigma=16 in, complex
-    FP32 out: one persistent launch (C >= 2048 tiles on whole CTAs, C <= 1024 tiles on
+    FP32 out: one persistent launch (C >= 1024 tiles on whole CTAs, C <= 512 tiles on
     half-CTA groups), replayed from a CUDA graph after autotuning."""
     import numpy as np
     import torch

@@ -29,8 +29,8 @@
 // T = 64; the FIR takes 1.8 there with two warps per scheduler, the DFT 0.6.
 // Against the form it replaces (channel pairs, batches of 16, taps and rows
 // requested by consumer threads; GS/s, 2^27 samples): C = 512 FP32 T = 64 90 ->
-// 137, T = 32 133 -> 188; int8 98 -> 140, 159 -> 203; C = 128 FP32 T = 32 114 -> 204;
-// C = 64 int8 T = 40 139 -> 170.  Also tried: taps through registers 8 ahead
+// 136, T = 32 133 -> 188; int8 98 -> 141, 159 -> 206; C = 128 FP32 T = 32 114 -> 204;
+// C = 64 int8 T = 40 139 -> 178.  Also tried: taps through registers 8 ahead
 // (the loads' latency shows: 58 GS/s at T = 64), in two sets of 8 registers
 // (spills: 116), refills by the last warp off a slot (73).
 #pragma once

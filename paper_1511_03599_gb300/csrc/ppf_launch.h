@@ -11,7 +11,7 @@ namespace ppf {
 // (grid_dependency_wait, the first thing such a kernel does, before any access
 // to memory).  Saves about 2 us between back-to-back launches (64 spectra at
 // C = 512: 6.15 -> 4.6 us per call).  Plain stream order while the stream is
-// being captured.
+// being captured: a replayed graph does without the saving.
 template <class K, class... A>
 inline cudaError_t launch_early(K kernel, dim3 grid, dim3 block, int smem, cudaStream_t st, const A&... args) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
