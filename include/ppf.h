@@ -287,7 +287,7 @@ const char* ppf_last_error_message(void);
  *   batches; bit 4: thread-block-cluster kernel, info[2] then counts the
  *   CTAs of whole clusters; bit 6: long-tap
  *   kernel, T = 17..64, raw rows and halo streamed through a TMA ring;
- *   bit 7: row kernel, C >= 1024 and C = 3*2^k, whose short calls
+ *   bit 7: row kernel, C >= 1024 and C = 3*2^k, whose short calls and streams
  *   run on batches of about a quarter of info[1]),
  *   info[7]=CTAs resident per SM. */
 ppf_status ppf_plan_info(ppf_plan_t plan, int info[8]);
